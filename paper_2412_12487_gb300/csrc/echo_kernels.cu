@@ -3,6 +3,7 @@
 // round-to-nearest intrinsics (no contraction), so results do not depend on -fmad.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -148,26 +149,88 @@ __global__ void cc_query_kernel(int64_t n, const uint8_t *__restrict__ type, con
 // load: caller-order rows -> internal order and blocked layout, with validation
 // and per-scenario sums
 // ---------------------------------------------------------------------------------
+// What bounds it is memory.  Three things had to go for that (GPT-1.3B x 256, int64):
+//   - an fp64 conversion and addition per element for the sums (140 us by the part's fp64
+//     rate of 527 G/s): they are exact integers, in halves of 32 bits, until the end;
+//   - an fp64 atomic per thread at the end (2 M of them): one per column and block;
+//   - rows of 8 to 128 bytes stored one by one in narrow blocks: a tile of kTileOps rows x
+//     kTileCols scenarios goes through shared memory, so that neighbouring rows of a block
+//     are stored together; the next tile is loaded meanwhile (185 us without that, 97 with).
+// 158 us before in blocks of 32 scenarios, 270 us in blocks of 2; 97 us in both (6.1 of the
+// 6.8 TB/s of a copy).
+constexpr int kTileLog = 5, kTileOps = 1 << kTileLog, kTileCols = 64;
 template <typename T>
-__global__ void permute_rows_kernel(const T *__restrict__ raw, const int32_t *__restrict__ int2ext,
-                                    const uint8_t *__restrict__ local, int64_t V, int32_t S, MatLayout lay,
-                                    int64_t *__restrict__ dur, double *__restrict__ sums, int32_t *status) {
-  int32_t s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= S) return;
-  double acc = 0.0;
+__global__ void __launch_bounds__(256, 6) permute_rows_kernel(const T *__restrict__ raw, const int32_t *__restrict__ int2ext,
+                                                              const uint8_t *__restrict__ local, int64_t V, int32_t S,
+                                                              MatLayout lay, int64_t *__restrict__ dur,
+                                                              double *__restrict__ sums, int32_t *status) {
+  constexpr int kGroups = 256 / kTileCols, kEach = kTileOps / kGroups;  // rows a thread loads of a tile
+  __shared__ T tile[kTileOps][kTileCols + 1];
+  // the caller's row, -1: a comm op's (0 until the collectives are estimated)
+  __shared__ int32_t from[2][kTileOps];
+  const int col = threadIdx.x % kTileCols, grp = threadIdx.x / kTileCols;
+  const int32_t c0 = blockIdx.x * kTileCols, s = c0 + col;
+  const int sl = lay.slog2, pl = kTileLog + sl;  // (log2 of) a row's scenarios in a block, the tile's elements in one
+  uint64_t lo = 0;
+  int64_t hi = 0;
   bool neg = false;
-  for (int64_t i = blockIdx.y; i < V; i += gridDim.y) {
-    int64_t e = int2ext[i];
-    int64_t d = 0;
-    if (local[i]) {
-      d = (int64_t)raw[e * S + s];
-      neg |= d < 0;
-      acc += (double)d;
+  // while a tile is stored, the next one's elements are on their way, and the places of
+  // the one after that (two dependent loads)
+  const int64_t step = (int64_t)gridDim.y * kTileOps, first = (int64_t)blockIdx.y * kTileOps;
+  auto rows = [&](int64_t i0, int b) {
+    if (threadIdx.x < kTileOps) {
+      const int64_t i = i0 + threadIdx.x;
+      from[b][threadIdx.x] = i < V && local[i] ? int2ext[i] : -1;
     }
-    dur[lay.at(i, s)] = d;
+  };
+  T x[kEach];
+  auto load = [&](int b) {
+#pragma unroll
+    for (int k = 0; k < kEach; ++k) {
+      const int32_t e = from[b][k * kGroups + grp];
+      x[k] = s < S && e >= 0 ? raw[(int64_t)e * S + s] : 0;
+    }
+  };
+  rows(first, 0);
+  __syncthreads();
+  load(0);
+  rows(first + step, 1);
+  __syncthreads();
+  int b = 1;
+  for (int64_t i0 = first; i0 < V; i0 += step, b ^= 1) {
+#pragma unroll
+    for (int k = 0; k < kEach; ++k) {
+      neg |= x[k] < 0;
+      lo += (uint32_t)x[k];
+      if (sizeof(T) == 8) hi += (int64_t)x[k] >> 32;
+      tile[k * kGroups + grp][col] = x[k];
+    }
+    load(b);
+    rows(i0 + 2 * step, b ^ 1);
+    __syncthreads();
+    const int n = (int)min((int64_t)kTileOps, V - i0);
+#pragma unroll
+    for (int k = 0; k < kEach; ++k) {
+      const int e = k * 256 + threadIdx.x, blk = e >> pl, y = e & ((1 << pl) - 1);
+      const int o = y >> sl, c = (blk << sl) + (y & ((1 << sl) - 1));
+      if (o < n && c0 + c < S) dur[lay.at(i0 + o, c0 + c)] = (int64_t)tile[o][c];
+    }
+    __syncthreads();
   }
   if (neg) set_status(status, kDevNegativeDuration);
-  atomicAdd(&sums[s], acc);
+  // one atomic per column and block
+  __shared__ uint64_t lo_s[256];
+  __shared__ int64_t hi_s[256];
+  lo_s[threadIdx.x] = lo;
+  hi_s[threadIdx.x] = hi;
+  __syncthreads();
+  if (grp == 0 && s < S) {
+    for (int k = kTileCols; k < 256; k += kTileCols) {
+      lo += lo_s[k + col];
+      hi += hi_s[k + col];
+    }
+    atomicAdd(&sums[s], (double)lo + (double)hi * 4294967296.0);
+  }
 }
 
 // ---------------------------------------------------------------------------------
@@ -296,16 +359,15 @@ cudaError_t launch_permute_rows(const void *raw, int bits, const int32_t *int2ex
                                 int32_t S, MatLayout lay, int64_t *dur, double *sums, int32_t *status,
                                 cudaStream_t st) {
   if (V == 0 || S == 0) return cudaSuccess;
-  int tx = S >= 128 ? 128 : ((S + 31) / 32) * 32;
-  dim3 block(tx);
-  int64_t gy = V < 8192 ? V : 8192;
-  dim3 grid((S + tx - 1) / tx, (unsigned)gy);
+  // one wave of blocks: 6 of 256 threads on an SM
+  const int64_t cols = (S + kTileCols - 1) / kTileCols, tiles = (V + kTileOps - 1) / kTileOps;
+  const dim3 grid((unsigned)cols, (unsigned)std::min<int64_t>(tiles, std::max<int64_t>(1, 152 * 6 / cols)));
   if (bits == 32)
-    permute_rows_kernel<int32_t><<<grid, block, 0, st>>>(static_cast<const int32_t *>(raw), int2ext, local, V, S,
-                                                         lay, dur, sums, status);
+    permute_rows_kernel<int32_t><<<grid, 256, 0, st>>>(static_cast<const int32_t *>(raw), int2ext, local, V, S, lay, dur,
+                                                       sums, status);
   else
-    permute_rows_kernel<int64_t><<<grid, block, 0, st>>>(static_cast<const int64_t *>(raw), int2ext, local, V, S,
-                                                         lay, dur, sums, status);
+    permute_rows_kernel<int64_t><<<grid, 256, 0, st>>>(static_cast<const int64_t *>(raw), int2ext, local, V, S, lay, dur,
+                                                       sums, status);
   return cudaGetLastError();
 }
 
