@@ -2141,6 +2141,17 @@ static int composition_status(echo_ctx *c) {
   return ECHO_OK;
 }
 
+// NULL, or plain memory of the context's device.
+static bool device_buffer(echo_ctx *c, const void *p) {
+  if (!p) return true;
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == c->device && (reinterpret_cast<uintptr_t>(p) & 7) == 0;
+}
+
 static int read_range_check(echo_ctx *c, int64_t op0, int64_t op1, int need_state) {
   if (c->state < need_state) return set_err(c, ECHO_E_STATE, "nothing to read yet");
   if (op0 < 0 || op1 < op0 || op1 > c->gb.V_ext) return set_err(c, ECHO_E_INVALID_ARG, "op range out of bounds");
@@ -2157,6 +2168,16 @@ int echo_read_times(echo_ctx *c, int64_t op0, int64_t op1, int32_t s0, int32_t s
   if ((rc = composition_status(c))) return rc;
   const int32_t Sr = s1 - s0;
   if (Sr == 0) return ECHO_OK;
+  // Buffers of this device are written to directly: through the staging buffer every value
+  // was written and read once more (GPT-175B x 250: 1.3 of 3.2 ms).
+  if (device_buffer(c, start) && device_buffer(c, finish)) {
+    CK(timed(c, "readback", [&] {
+         return echo::launch_readback(c->ext2int, op0, op1, s0, s1, c->lay, c->f[c->final_f], c->dur, c->cidx, c->lay_c,
+                                      c->final_cd, start, finish, c->stream);
+       }), "readback launch");
+    CK(cudaStreamSynchronize(c->stream), "readback");
+    return ECHO_OK;
+  }
   const int64_t rows_per = std::max<int64_t>(1, (int64_t)(64 << 20) / Sr);
   if ((rc = stage_reserve(c, (size_t)std::min<int64_t>(rows_per, std::max<int64_t>(op1 - op0, 1)) * Sr * 16)))
     return rc;

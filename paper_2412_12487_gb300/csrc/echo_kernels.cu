@@ -279,6 +279,78 @@ __global__ void readback_kernel(const int32_t *__restrict__ ext2int, int64_t op0
   }
 }
 
+// The same for whole batches (32 scenarios and more) in narrow blocks, where a row of one
+// block is only 8 to 128 bytes.  What bounds it is memory: a tile of kTileOps ops x
+// kReadCols scenarios goes through shared memory, so that the loads take neighbouring rows
+// of a block together (ops of a chain are neighbours in both orders) and the stores whole
+// rows of the caller's; a tile is loaded while the one before it is stored.
+constexpr int kReadCols = 32;
+__global__ void __launch_bounds__(256, 4) readback_tile_kernel(
+    const int32_t *__restrict__ ext2int, int64_t op0, int64_t op1, int32_t s0, int32_t s1, MatLayout lay,
+    const int64_t *__restrict__ f, const int64_t *__restrict__ d, const int32_t *__restrict__ cidx, MatLayout lay_c,
+    const int64_t *__restrict__ cd, int64_t *__restrict__ start, int64_t *__restrict__ finish) {
+  constexpr int kEach = kTileOps * kReadCols / 256;
+  // (rows padded by one element: a warp's column of them falls into different banks)
+  __shared__ int64_t ft[kTileOps][kReadCols + 1], st[kTileOps][kReadCols + 1];
+  __shared__ int32_t row[2][kTileOps], crow[2][kTileOps];
+  const int32_t c0 = (s0 & ~(kReadCols - 1)) + blockIdx.y * kReadCols;  // first scenario of the tile
+  const int sl = lay.slog2, pl = kTileLog + sl;  // (log2 of) a row's scenarios in a block, the tile's elements in one
+  const int64_t step = (int64_t)gridDim.x * kTileOps, first = op0 + (int64_t)blockIdx.x * kTileOps;
+  auto rows = [&](int64_t o0, int b) {
+    if (threadIdx.x < kTileOps) {
+      const int64_t o = o0 + threadIdx.x;
+      const int32_t i = o < op1 ? ext2int[o] : -1;
+      row[b][threadIdx.x] = i;
+      crow[b][threadIdx.x] = cd && i >= 0 ? cidx[i] : -1;
+    }
+  };
+  int64_t fv[kEach], dv[kEach];
+  auto load = [&](int b) {
+#pragma unroll
+    for (int k = 0; k < kEach; ++k) {
+      const int e = k * 256 + threadIdx.x, blk = e >> pl, y = e & ((1 << pl) - 1);
+      const int o = y >> sl, s = c0 + (blk << sl) + (y & ((1 << sl) - 1));
+      const int32_t i = row[b][o], ci = crow[b][o];
+      fv[k] = dv[k] = 0;
+      if (i >= 0 && s >= s0 && s < s1) {
+        const int64_t at = lay.at(i, s);
+        fv[k] = f[at];
+        if (start) dv[k] = ci >= 0 ? cd[lay_c.at(ci, s)] : d[at];
+      }
+    }
+  };
+  rows(first, 0);
+  __syncthreads();
+  load(0);
+  rows(first + step, 1);
+  __syncthreads();
+  const int64_t Sr = s1 - s0;
+  int b = 1;
+  for (int64_t o0 = first; o0 < op1; o0 += step, b ^= 1) {
+#pragma unroll
+    for (int k = 0; k < kEach; ++k) {
+      const int e = k * 256 + threadIdx.x, blk = e >> pl, y = e & ((1 << pl) - 1);
+      const int o = y >> sl, c = (blk << sl) + (y & ((1 << sl) - 1));
+      ft[o][c] = fv[k];
+      st[o][c] = fv[k] - dv[k];
+    }
+    load(b);
+    rows(o0 + 2 * step, b ^ 1);
+    __syncthreads();
+    const int n = (int)min((int64_t)kTileOps, op1 - o0);
+#pragma unroll
+    for (int k = 0; k < kEach; ++k) {
+      const int e = k * 256 + threadIdx.x, o = e / kReadCols, c = e % kReadCols, s = c0 + c;
+      if (o < n && s >= s0 && s < s1) {
+        const int64_t to = (o0 - op0 + o) * Sr + (s - s0);
+        if (finish) finish[to] = ft[o][c];
+        if (start) start[to] = st[o][c];
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // Full validator durations for the kernels without a candidate ring: the
 // candidates' rows of the compact cd into dst (which holds the original durations).
 __global__ void scatter_candidates_kernel(const int32_t *__restrict__ cand_node, int64_t n_cand, int32_t S,
@@ -417,6 +489,14 @@ cudaError_t launch_readback(const int32_t *ext2int, int64_t op0, int64_t op1, in
                             const int64_t *cd, int64_t *start, int64_t *finish, cudaStream_t st) {
   int64_t n = (op1 - op0) * (s1 - s0);
   if (n <= 0) return cudaSuccess;
+  if (s1 - s0 >= kReadCols && lay.slog2 < 5) {
+    const int32_t first = s0 & ~(kReadCols - 1);
+    const int64_t cols = (s1 - first + kReadCols - 1) / kReadCols, tiles = (op1 - op0 + kTileOps - 1) / kTileOps;
+    // one wave of blocks: 4 of 256 threads on an SM
+    const dim3 grid((unsigned)std::min<int64_t>(tiles, std::max<int64_t>(1, 152 * 4 / cols)), (unsigned)cols);
+    readback_tile_kernel<<<grid, 256, 0, st>>>(ext2int, op0, op1, s0, s1, lay, f, d, cidx, lay_c, cd, start, finish);
+    return cudaGetLastError();
+  }
   readback_kernel<<<grid_for(n, 256), 256, 0, st>>>(ext2int, op0, op1, s0, s1, lay, f, d, cidx, lay_c, cd, start,
                                                     finish);
   return cudaGetLastError();
