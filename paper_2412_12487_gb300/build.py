@@ -19,7 +19,7 @@ INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG, "libecho.so")
 BUILD_DIR = os.path.join(PKG, "_build")
 # (source, extra nvcc flags, object)
-UNITS = [(f, [], f + ".o") for f in ("echo_kernels.cu", "echo_compose.cu", "echo_dataflow.cu", "echo_host.cpp")] + [
+UNITS = [(f, [], f + ".o") for f in ("echo_kernels.cu", "echo_compose.cu", "echo_levels.cu", "echo_dataflow.cu", "echo_host.cpp")] + [
     ("echo_overlap.cu", [f"-DECHO_OV_LAUNCH={l}", f"-DECHO_OV_PROP={p}"], f"echo_overlap_l{l}_p{p}.o")
     for l in (0, 1) for p in (0, 1)]
 SOURCES = sorted({u[0] for u in UNITS})

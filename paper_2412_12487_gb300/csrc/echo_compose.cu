@@ -23,7 +23,8 @@ namespace {
 // per-scenario makespan is fused in.
 //
 // compose_direct_kernel reads the graph and the durations from global memory and
-// fits any graph; the staged and pipelined kernels are the fast paths.
+// fits any graph; the staged kernel streams both through shared memory.  The fast
+// path is compose_levels_kernel (echo_levels.cu).
 // ---------------------------------------------------------------------------------
 template <int SIGMA, bool SMEM_FRONTIER>
 __global__ void __launch_bounds__(kComposeThreads)
@@ -182,13 +183,12 @@ __device__ __forceinline__ void g_store(int64_t *p, const int64_t (&v)[LANES]) {
     *p = v[0];
 }
 
-// Debug bounds (out of line, off the hot path): the segment's chain rows, its
-// candidates' compact rows, every input's value-ring slot and far row.  A failed
-// check records kDevBounds.
-__device__ __noinline__ bool segment_ok(const StagedArgs &a, uint32_t first, uint32_t len, uint64_t cmask,
-                                        uint32_t c_first, uint32_t rr_a, uint32_t rmask, uint32_t e, uint32_t nin,
-                                        uint32_t nfar, uint32_t ring_bytes, uint32_t row_bytes) {
-  bool ok = len > 0 && range_ok(first, (int64_t)first + len, a.n_rows) && masked_row_ok(c_first, cmask, a.n_cand);
+// Debug bounds (out of line, off the hot path): the segment's chain rows, every
+// input's value-ring slot and far row.  A failed check records kDevBounds.
+__device__ __noinline__ bool segment_ok(const StagedArgs &a, uint32_t first, uint32_t len, uint32_t rr_a,
+                                        uint32_t rmask, uint32_t e, uint32_t nin, uint32_t nfar, uint32_t ring_bytes,
+                                        uint32_t row_bytes) {
+  bool ok = len > 0 && range_ok(first, (int64_t)first + len, a.n_rows);
   for (uint32_t x = 0; ok && x < nin + nfar; ++x) {
     uint32_t w;
     asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(w) : "r"(rr_a + ((e + x) & rmask) * 4));
@@ -198,12 +198,10 @@ __device__ __noinline__ bool segment_ok(const StagedArgs &a, uint32_t first, uin
   return ok;
 }
 
-// Compose the segments of one segment level (shared by the staged and the
-// pipelined kernels).  Segment k's header and entries are in the record ring at
-// word `ro`; its rows are i0 + header.z ... (global rows), held in the duration
-// ring of RR rows from ring row dpos0 + header.z on (wrapping).  Candidate rows of
-// the level start at level-order index c0, in ring row cpos0 of the CRR-row
-// candidate ring.  Thread `sub` handles segments sub, sub + step, ... for scenario
+// Compose the segments of one segment level.  Segment k's header and entries are in
+// the record ring at word `ro`; its rows are i0 + header.z ... (global rows), held in
+// the duration ring of RR rows (a power of two) from ring row dpos0 + header.z on
+// (wrapping).  Thread `sub` handles segments sub, sub + step, ... for scenario
 // lanes j0 .. j0+LANES-1; the segments of a level come heaviest first, so a warp's
 // lanes hold segments of similar weight.  Every input of a head is the tail of an earlier segment: the
 // recent ones are read from the value ring (entries are byte offsets of their
@@ -215,51 +213,30 @@ template <int SIGMA, int LANES, bool STORE_ALL, bool DBG>
 __device__ __forceinline__ void compose_segments(const StagedArgs &a, uint32_t ro, uint32_t i0, uint32_t seg0,
                                                  int32_t nseg, int sub, int step, int j0, int64_t *vr,
                                                  const int64_t *dr, const uint32_t *rr, uint32_t vmask,
-                                                 uint32_t dpos0, uint32_t RR, uint32_t rmask, int64_t (&mk)[LANES],
-                                                 const int64_t *cr = nullptr, uint32_t cpos0 = 0, uint32_t c0 = 0,
-                                                 uint32_t CRR = 0) {
-  int64_t *fb = a.f + ((int64_t)blockIdx.x * a.n_rows) * SIGMA;
+                                                 uint32_t dpos0, uint32_t RR, uint32_t rmask, int64_t (&mk)[LANES]) {
+  int64_t *fb = a.f + ((int64_t)blockIdx.x * a.pitch) * SIGMA;
   const uint32_t vr_a = saddr(vr) + j0 * 8, dr_a = saddr(dr) + j0 * 8;
   const uint32_t rr_a = saddr(rr);
-  const uint32_t cr_a = cr ? saddr(cr) + j0 * 8 : 0;
   constexpr uint32_t kRowBytes = SIGMA * 8;
   auto word = [&](uint32_t w) { return s_ld32(rr_a + (w & rmask) * 4); };
   for (int32_t k = sub; k < nseg; k += step) {
     const uint4 hd = s_ld128(rr_a + ((ro + 4 * k) & rmask) * 4);
     const uint32_t nin = hd.y & 0xFFFFu, nfar = hd.y >> 16;
     const uint32_t len = hd.w & 0xFFFFu;
-    // chain positions whose duration the validator rewrote (second and later passes)
-    const bool has_c = (hd.w >> 16) & 1, has_k = (hd.w >> 17) & 1;
-    const uint32_t ec = ro + hd.x + nin + nfar;
-    uint64_t cmask_bits = 0;
-    uint32_t c_first = 0;
-    if (cr && has_c) {
-      cmask_bits = (uint64_t)word(ec) | ((uint64_t)word(ec + 1) << 32);
-      c_first = word(ec + 2);
-    }
+    const bool has_k = (hd.w >> 17) & 1;
     // chain positions whose finish is stored: all in the final composition; else
     // the tail (later heads read it) and those a later step reads (kept mask)
     uint64_t smask = ~0ull;
     if (!STORE_ALL) {
       smask = 1ull << (len - 1);
       if (has_k) {
-        const uint32_t ek = ec + (has_c ? 3 : 0);
+        const uint32_t ek = ro + hd.x + nin + nfar;
         smask |= (uint64_t)word(ek) | ((uint64_t)word(ek + 1) << 32);
       }
     }
-    // a candidate's duration comes from the candidate ring instead of the duration ring
-    // (the level's candidates span at most CRR rows, so one wrap suffices)
-    auto patch = [&](uint32_t t, int64_t (&d)[LANES]) {
-      if ((cmask_bits >> t) & 1) {
-        uint32_t x = cpos0 + (c_first - c0) + (uint32_t)__popcll(cmask_bits & ((1ull << t) - 1));
-        if (x >= CRR) x -= CRR;
-        s_load<LANES>(cr_a + x * kRowBytes, d);
-      }
-    };
     const uint32_t e = ro + hd.x;
     const uint32_t first = i0 + hd.z;
-    if (DBG && !segment_ok(a, first, len, cmask_bits, c_first, rr_a, rmask, e, nin, nfar, (vmask + 1) * kRowBytes,
-                             kRowBytes))
+    if (DBG && !segment_ok(a, first, len, rr_a, rmask, e, nin, nfar, (vmask + 1) * kRowBytes, kRowBytes))
       continue;  // debug bounds: a bad index skips the segment
     int64_t fv[LANES];
 #pragma unroll
@@ -296,12 +273,6 @@ __device__ __forceinline__ void compose_segments(const StagedArgs &a, uint32_t r
       s_load<LANES>(dr_a + p2 * kRowBytes, d2);
       s_load<LANES>(dr_a + p3 * kRowBytes, d3);
       p = next(p3);
-      if (cmask_bits) {
-        patch(t, d0);
-        patch(t + 1, d1);
-        patch(t + 2, d2);
-        patch(t + 3, d3);
-      }
       const uint32_t sb = (uint32_t)(smask >> t);
 #pragma unroll
       for (int j = 0; j < LANES; ++j) fv[j] += d0[j];
@@ -319,7 +290,6 @@ __device__ __forceinline__ void compose_segments(const StagedArgs &a, uint32_t r
     for (; t < len; ++t, gp += SIGMA, p = next(p)) {
       int64_t d[LANES];
       s_load<LANES>(dr_a + p * kRowBytes, d);
-      if (cmask_bits) patch(t, d);
 #pragma unroll
       for (int j = 0; j < LANES; ++j) fv[j] += d[j];
       if (STORE_ALL || ((smask >> t) & 1)) g_store<LANES>(gp, fv);
@@ -351,7 +321,7 @@ compose_staged_kernel(StagedArgs a) {
   const int tid = threadIdx.x;
   const uint32_t vmask = (1u << a.vlog2) - 1, dmask = (1u << a.dlog2) - 1, rmask = (1u << a.rlog2) - 1;
   const uint32_t RR = dmask + 1, RB = rmask + 1;
-  const StagedLayout lay = staged_layout(SIGMA, a.vlog2, RR, a.rlog2, (size_t)1 << a.clog2);
+  const StagedLayout lay = staged_layout(SIGMA, a.vlog2, RR, a.rlog2);
   int64_t *mk_s = reinterpret_cast<int64_t *>(sbuf);                  // [SIGMA]
   uint2 *hist = reinterpret_cast<uint2 *>(sbuf + lay.hist);           // [16] (rows, words) copied by group
   uint32_t *meta_s = reinterpret_cast<uint32_t *>(sbuf + lay.meta);   // [2][kMetaCap][4]
@@ -368,7 +338,7 @@ compose_staged_kernel(StagedArgs a) {
   };
   // this block's rows are contiguous: element e of the block lands in ring element
   // e mod (RR*SIGMA), and a 16-byte piece never straddles the ring's end
-  const int64_t *durb = a.dur + ((int64_t)blockIdx.x * a.n_rows) * SIGMA;
+  const int64_t *durb = a.dur + ((int64_t)blockIdx.x * a.pitch) * SIGMA;
   const uint32_t emask = RR * SIGMA - 1;
   uint32_t rows_done = 0, words_done = 0;
   auto issue_to = [&](uint32_t row_lim, uint32_t word_lim) {  // copy rows and words up to the limits
@@ -449,194 +419,6 @@ compose_staged_kernel(StagedArgs a) {
   if (tid < SIGMA && s0 + tid < S && a.makespan) a.makespan[s0 + tid] = mk_s[tid];
 }
 
-// -- mbarriers and 1-D bulk copies (TMA engine) ----------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
-// wait for the phase of `parity` to complete; false once `limit` clock cycles pass
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, long long limit) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity))
-    if (clock64() - t0 > limit) return false;
-  return true;
-}
-// addresses 16-byte aligned, size a multiple of 16; completes `bytes` on the mbarrier
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-// barrier over `threads` threads that also returns whether any of them passed `flag`
-__device__ __forceinline__ bool named_barrier_or(int id, int threads, bool flag) {
-  uint32_t any;
-  asm volatile(
-      "{\n .reg .pred pin, pout;\n setp.ne.u32 pin, %1, 0;\n bar.red.or.pred pout, %2, %3, pin;\n"
-      " selp.u32 %0, 1, 0, pout;\n}\n"
-      : "=r"(any) : "r"((uint32_t)flag), "r"(id), "r"(threads) : "memory");
-  return any != 0;
-}
-
-// Pipelined compose (even SIGMA): the last warp is a producer that copies each
-// segment level's duration rows, record block and metadata into the rings with the
-// TMA engine (at most five 1-D bulk copies per level: this block's rows of a level
-// are contiguous), as far ahead as the rings allow; kPipeConsumerWarps warps
-// compose, one scenario per thread up to SIGMA 8 (a segment's SIGMA threads
-// share its walk), two above.  The duration and candidate rings hold any number
-// of rows (a.d_rows, a.c_rows: all the shared memory the rest leaves), so the
-// producer writes each level's first ring rows beside its metadata.  Stage
-// l % kPipeStages has a "full" mbarrier (armed with the level's byte count) and
-// an "empty" mbarrier (one arrival per consumer warp once the level is composed).  Every wait is bounded: on expiry the block records
-// kDevTimeout, stops, and lets its copies in flight land first.
-template <int SIGMA, bool STORE_ALL, bool DBG>
-__global__ void __launch_bounds__((kPipeConsumerWarps + 1) * 32)
-compose_pipelined_kernel(StagedArgs a) {
-  constexpr int LANES = SIGMA <= 8 ? 1 : 2;
-  constexpr int TPN = SIGMA / LANES;  // threads per segment
-  constexpr int NB = kPipeStages;
-  constexpr int NCT = kPipeConsumerWarps * 32;
-  extern __shared__ __align__(16) unsigned char sbuf[];
-  const int32_t S = a.S;
-  const int32_t s0 = blockIdx.x * SIGMA;
-  const int tid = threadIdx.x;
-  const StagedLayout lay = staged_layout(SIGMA, a.vlog2, a.d_rows, a.rlog2, a.c_rows);
-  const uint32_t vmask = (1u << a.vlog2) - 1, rmask = (1u << a.rlog2) - 1;
-  const uint32_t RR = a.d_rows, RB = rmask + 1, CRR = a.c_rows;
-  int64_t *mk_s = reinterpret_cast<int64_t *>(sbuf);                       // [SIGMA]
-  uint64_t *full = reinterpret_cast<uint64_t *>(sbuf + lay.meta);          // [NB]
-  uint64_t *empty = full + NB;                                              // [NB]
-  uint32_t *hist = reinterpret_cast<uint32_t *>(sbuf + lay.meta + 256);    // [NB][4] producer only
-  uint32_t *metas = reinterpret_cast<uint32_t *>(sbuf + lay.meta + 512);   // [NB][8]
-  uint32_t *pos = reinterpret_cast<uint32_t *>(sbuf + lay.meta + 1024);    // [NB][2] first ring rows
-  int64_t *vr = reinterpret_cast<int64_t *>(sbuf + lay.vr);
-  int64_t *dr = reinterpret_cast<int64_t *>(sbuf + lay.dr);
-  uint32_t *rr = reinterpret_cast<uint32_t *>(sbuf + lay.rr);
-  int64_t *cr = reinterpret_cast<int64_t *>(sbuf + lay.cr);
-
-  if (tid < SIGMA) mk_s[tid] = 0;
-  if (tid == 0) {
-    for (int b = 0; b < NB; ++b) {
-      mbar_init(&full[b], 1);  // the producer's arrive.expect_tx
-      mbar_init(&empty[b], kPipeConsumerWarps);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  __syncthreads();
-
-  if (tid >= NCT) {
-    // ---------------- producer warp (one lane issues) ----------------
-    const int lane = tid - NCT;
-    if (lane == 0) {
-      const int64_t *durb = a.dur + ((int64_t)blockIdx.x * a.n_rows) * SIGMA;
-      const int64_t *cdb = a.cdur ? a.cdur + ((int64_t)blockIdx.x * a.n_cand) * SIGMA : nullptr;
-      int32_t c_known = 0;  // every level < c_known has been composed
-      int32_t issued = 0;   // levels [0, issued) have been armed
-      bool fail = false;
-      // metadata of levels l and l+1, and l+2 in flight (its load latency overlaps a level)
-      uint4 m_cur = *reinterpret_cast<const uint4 *>(a.meta);
-      uint4 m_nxt = *reinterpret_cast<const uint4 *>(a.meta + 4 * min(1, a.L));
-      for (int32_t l = 0; l < a.L; ++l) {
-        if (l == a.skip_level) break;  // failure injection: level l never arrives
-        const uint4 m_fut = *reinterpret_cast<const uint4 *>(a.meta + 4 * min(l + 2, a.L));
-        const uint4 m0 = m_cur, m1 = m_nxt;
-        m_cur = m_nxt;
-        m_nxt = m_fut;
-        uint32_t ro = m0.x, i0 = m0.y, ro1 = m1.x, i1 = m1.y;
-        uint32_t c0 = cdb ? m0.w : 0, c1 = cdb ? m1.w : 0;  // the level's candidate rows
-        if (DBG && !(range_ok(i0, i1, a.n_rows) && range_ok(ro, ro1, a.n_words) && range_ok(c0, c1, a.n_cand))) {
-          atomicCAS(a.status, 0, (int32_t)kDevBounds);  // debug bounds: copy nothing for this level
-          i1 = i0 = min(i0, a.n_rows);
-          ro1 = ro = min(ro, a.n_words);
-          c1 = c0 = min(c0, a.n_cand);
-        }
-        // ring space: level l overwrites rows and words of levels below c_known only
-        while (c_known < l && (l - c_known >= NB || i1 > hist[4 * (c_known % NB)] + RR ||
-                               ro1 > hist[4 * (c_known % NB) + 1] + RB || c1 > hist[4 * (c_known % NB) + 2] + CRR)) {
-          if (!mbar_wait(&empty[c_known % NB], (c_known / NB) & 1, a.wait_limit_cycles)) {
-            fail = true;
-            break;
-          }
-          ++c_known;
-        }
-        if (fail) break;
-        hist[4 * (l % NB)] = i0;
-        hist[4 * (l % NB) + 1] = ro;
-        hist[4 * (l % NB) + 2] = c0;
-        // ring rows of the level's first row and first candidate (read by the
-        // consumers after the level's full barrier, which this arrival releases)
-        const uint32_t dp = i0 % RR, cp = CRR ? c0 % CRR : 0;
-        pos[2 * (l % NB)] = dp;
-        pos[2 * (l % NB) + 1] = cp;
-        uint64_t *bar = &full[l % NB];
-        const uint32_t e0 = i0 * SIGMA, ne = (i1 - i0) * SIGMA, w0 = ro & rmask, nw = ro1 - ro;
-        const uint32_t ce0 = c0 * SIGMA, nce = (c1 - c0) * SIGMA;
-        mbar_arrive_expect_tx(bar, ne * 8 + nw * 4 + 32 + nce * 8);
-        if (nce) {
-          const uint32_t nce1 = min(nce, (CRR - cp) * SIGMA);
-          bulk_g2s(cr + cp * SIGMA, cdb + ce0, nce1 * 8, bar);
-          if (nce1 < nce) bulk_g2s(cr, cdb + ce0 + nce1, (nce - nce1) * 8, bar);
-        }
-        const uint32_t ne1 = min(ne, (RR - dp) * SIGMA);
-        bulk_g2s(dr + dp * SIGMA, durb + e0, ne1 * 8, bar);
-        if (ne1 < ne) bulk_g2s(dr, durb + e0 + ne1, (ne - ne1) * 8, bar);
-        const uint32_t nw1 = min(nw, RB - w0);
-        bulk_g2s(rr + w0, a.recs + ro, nw1 * 4, bar);
-        if (nw1 < nw) bulk_g2s(rr, a.recs + ro + nw1, (nw - nw1) * 4, bar);
-        bulk_g2s(metas + 8 * (l % NB), a.meta + 4 * l, 32, bar);
-        issued = l + 1;
-      }
-      if (fail) atomicCAS(a.status, 0, kDevTimeout);
-      // let every copy this block started land before it exits
-      for (int32_t x = max(c_known, issued - NB); x < issued; ++x)
-        if (!mbar_wait(&full[x % NB], (x / NB) & 1, a.wait_limit_cycles)) atomicCAS(a.status, 0, kDevTimeout);
-    }
-    __syncwarp();
-  } else {
-    // ---------------- consumer warps ----------------
-    const int j0 = (tid % TPN) * LANES;
-    int64_t mk[LANES];
-#pragma unroll
-    for (int j = 0; j < LANES; ++j) mk[j] = 0;
-    for (int32_t l = 0; l < a.L; ++l) {
-      const bool ok = mbar_wait(&full[l % NB], (l / NB) & 1, a.wait_limit_cycles);
-      if (ok) {
-        const uint32_t *mb = metas + 8 * (l % NB);
-        const uint32_t ro = mb[0], i0 = mb[1], seg0 = mb[2], c0 = mb[3];
-        const int32_t nseg = (int32_t)(mb[4 + 2] - seg0);
-        const uint32_t dp = pos[2 * (l % NB)], cp = pos[2 * (l % NB) + 1];
-        compose_segments<SIGMA, LANES, STORE_ALL, DBG>(a, ro, i0, seg0, nseg, tid / TPN, NCT / TPN, j0, vr, dr,
-                                                       rr, vmask, dp, RR, rmask, mk, a.cdur ? cr : nullptr, cp,
-                                                       c0, CRR);
-      }
-      // every consumer learns, in the same barrier, whether any of them gave up
-      if (named_barrier_or(1, NCT, !ok)) {
-        if (tid == 0) atomicCAS(a.status, 0, kDevTimeout);
-        break;
-      }
-      if ((tid & 31) == 0) mbar_arrive(&empty[l % NB]);
-    }
-#pragma unroll
-    for (int j = 0; j < LANES; ++j) atomicMax((unsigned long long *)&mk_s[j0 + j], (unsigned long long)mk[j]);
-  }
-  __syncthreads();
-  if (tid < SIGMA && s0 + tid < S && a.makespan) a.makespan[s0 + tid] = mk_s[tid];
-}
-
 template <int SIGMA>
 cudaError_t launch_compose_t(const ComposeArgs &a, cudaStream_t st) {
   bool in_smem = false;
@@ -661,20 +443,6 @@ cudaError_t launch_staged_t(const StagedArgs &a, const StagedPlan &plan, cudaStr
   if (e != cudaSuccess) return e;
   dim3 grid((a.S + SIGMA - 1) / SIGMA);
   k<<<grid, THREADS, plan.smem, st>>>(a);
-  return cudaGetLastError();
-}
-
-template <int SIGMA>
-cudaError_t launch_pipelined_t(const StagedArgs &a, const StagedPlan &plan, cudaStream_t st) {
-  // debug bounds runs the checking variant, which stores every finish
-  auto k = a.dbg ? compose_pipelined_kernel<SIGMA, true, true>
-                 : a.store_all ? compose_pipelined_kernel<SIGMA, true, false> : compose_pipelined_kernel<SIGMA, false, false>;
-  (void)plan;
-  const size_t smem = staged_layout(SIGMA, a.vlog2, a.d_rows, a.rlog2, a.c_rows).total;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid((a.S + SIGMA - 1) / SIGMA);
-  k<<<grid, (kPipeConsumerWarps + 1) * 32, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -712,17 +480,6 @@ cudaError_t launch_compose_staged(const StagedArgs &a, int sigma, const StagedPl
     case 4 * 10000 + 512: return launch_staged_t<4, 512>(a, plan, st);
     case 8 * 10000 + 512: return launch_staged_t<8, 512>(a, plan, st);
     case 16 * 10000 + 1024: return launch_staged_t<16, 1024>(a, plan, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_compose_pipelined(const StagedArgs &a, int sigma, const StagedPlan &plan, cudaStream_t st) {
-  if (a.S == 0) return cudaSuccess;
-  switch (sigma) {
-    case 2: return launch_pipelined_t<2>(a, plan, st);
-    case 4: return launch_pipelined_t<4>(a, plan, st);
-    case 8: return launch_pipelined_t<8>(a, plan, st);
-    case 16: return launch_pipelined_t<16>(a, plan, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -83,6 +83,12 @@ struct GraphBuild {
   // chain: an overlap candidate, a comm op the validator's cursors visit, or one
   // of their launch conditions (a segment's tail is always kept: later heads read it)
   std::vector<uint8_t> keep;
+  std::vector<uint64_t> seg_keep, seg_cand;  // [n_seg] chain positions that are kept, that are candidates
+  // [n_seg] shared-memory slot of the tail's finish in the levelled composer (from 2 on; 1:
+  // no later head reads it), and their number: live from the segment's level to the last
+  // one that reads it, and given out again from the level after that on
+  std::vector<int32_t> seg_slot;
+  int64_t n_slots = 2;
   std::vector<int64_t> hin_off;       // [n_seg+1] inputs of each segment's head
   std::vector<int32_t> hin;           // (internal ids, each the tail of an earlier segment)
   int32_t max_kclass = -1;
@@ -617,18 +623,11 @@ int build_graph(const echo_graph_desc *g, GraphBuild &b, Err &e, const std::vect
   {
     std::vector<int64_t> cur(b.seg_lvl_off.begin(), b.seg_lvl_off.end() - 1);
     for (int64_t t = 0; t < NSg; ++t) seg_order[cur[seg_lvl[t]]++] = (int32_t)t;
-    // within a level the heaviest segments first (inputs and tail timelines weigh
-    // twice a chain step), so that a warp's lanes hold segments of similar weight
-    std::vector<int32_t> ntl(V, 0);
-    for (int64_t i = 0; i < QE; ++i) ntl[g->q_ops[i]]++;
-    std::vector<int64_t> cost(NSg);
-    for (int64_t t = 0; t < NSg; ++t) {
-      const int32_t h = seg_head[t], z = seg_tail[t];
-      cost[t] = 2 * (ntl[h] + (g->pred_off[h + 1] - g->pred_off[h]) + ntl[z]) + seg_len[t];
-    }
+    // within a level the longest segments first, so that a warp's lanes hold chains of
+    // similar length
     for (int64_t l = 0; l < Ls; ++l)
       std::stable_sort(seg_order.begin() + b.seg_lvl_off[l], seg_order.begin() + b.seg_lvl_off[l + 1],
-                       [&](int32_t x, int32_t y) { return cost[x] > cost[y]; });
+                       [&](int32_t x, int32_t y) { return seg_len[x] > seg_len[y]; });
   }
   // internal numbering: segment levels in order, each segment's chain contiguous
   b.seg_node_off.assign(NSg + 1, 0);
@@ -818,15 +817,21 @@ int build_graph(const echo_graph_desc *g, GraphBuild &b, Err &e, const std::vect
     for (int32_t q = b.lq_off[e]; q < b.lq_off[e + 1]; ++q) b.keep[b.lq_ops[q]] = 1;
   }
   b.seg_words.assign(NSg, 0);
+  b.seg_keep.assign(NSg, 0);
+  b.seg_cand.assign(NSg, 0);
   for (int64_t t = 0; t < NSg; ++t) {
     const int64_t nin = b.hin_off[t + 1] - b.hin_off[t];
     if (nin > 0xFFFF) b.stageable = false;
-    bool cand = false, kept = false;
-    for (int64_t v = b.seg_node_off[t]; v < b.seg_node_off[t + 1]; ++v) {
-      cand = cand || b.cand_flag[v];
-      kept = kept || (b.keep[v] && v + 1 < b.seg_node_off[t + 1]);
+    uint64_t keep = 0, cand = 0;
+    const int64_t v0 = b.seg_node_off[t], len = b.seg_node_off[t + 1] - v0;
+    for (int64_t i = 0; i < len; ++i) {
+      keep |= (uint64_t)b.keep[v0 + i] << i;
+      cand |= (uint64_t)b.cand_flag[v0 + i] << i;
     }
-    b.seg_words[t] = 4 + nin + (cand ? 3 : 0) + (kept ? 2 : 0);
+    b.seg_keep[t] = keep;
+    b.seg_cand[t] = cand;
+    const bool before_tail = keep & ((1ull << (len - 1)) - 1);  // the staged kernel always stores tails
+    b.seg_words[t] = 4 + nin + (before_tail ? 2 : 0);
   }
   // every input of a segment comes from an earlier level (the kernels' contract)
   {
@@ -838,6 +843,29 @@ int build_graph(const echo_graph_desc *g, GraphBuild &b, Err &e, const std::vect
         if (lvl[b.seg_int[b.hin[q]]] >= lvl[t])
           return fail(e, ECHO_E_BAD_GRAPH, "internal: segment %lld reads level %d from level %d", (long long)t,
                       lvl[b.seg_int[b.hin[q]]], lvl[t]);
+    if (programs) {
+      std::vector<int32_t> last(NSg, -1), freed, next(NSg, -1), head(Ls, -1);  // head, next: tails by the level that reads them last
+      for (int64_t t = 0; t < NSg; ++t)
+        for (int64_t q = b.hin_off[t]; q < b.hin_off[t + 1]; ++q) last[b.seg_int[b.hin[q]]] = lvl[t];  // (t ascends by level)
+      for (int64_t t = 0; t < NSg; ++t)
+        if (last[t] >= 0) {
+          next[t] = head[last[t]];
+          head[last[t]] = (int32_t)t;
+        }
+      b.seg_slot.assign(NSg, 1);
+      for (int64_t l = 0; l < Ls; ++l) {
+        for (int64_t t = b.seg_lvl_off[l]; t < b.seg_lvl_off[l + 1]; ++t) {
+          if (last[t] < 0) continue;
+          if (freed.empty()) {
+            b.seg_slot[t] = (int32_t)b.n_slots++;
+          } else {
+            b.seg_slot[t] = freed.back();
+            freed.pop_back();
+          }
+        }
+        for (int32_t t = head[l]; t >= 0; t = next[t]) freed.push_back(b.seg_slot[t]);
+      }
+    }
   }
   if (programs) build_dataflow(b);
   return ECHO_OK;
@@ -1105,7 +1133,6 @@ struct Steps {
   int64_t L = 0;
   std::vector<int64_t> off;    // [L+1] segments of each step
   std::vector<int64_t> words;  // [L] record block words (padded to 4)
-  std::vector<int64_t> cand;   // [L+1] first level-order candidate of each step
 };
 
 Steps make_steps(const GraphBuild &b, int64_t cap) {
@@ -1123,13 +1150,10 @@ Steps make_steps(const GraphBuild &b, int64_t cap) {
   }
   st.L = (int64_t)st.off.size() - 1;
   st.words.assign(st.L, 0);
-  st.cand.assign(st.L + 1, b.n_cand);
   for (int64_t l = 0; l < st.L; ++l) {
     int64_t w = 0;
     for (int64_t t = st.off[l]; t < st.off[l + 1]; ++t) w += b.seg_words[t];
     st.words[l] = (w + 3) & ~(int64_t)3;
-    const int32_t first = (int32_t)b.seg_node_off[st.off[l]];
-    st.cand[l] = std::lower_bound(b.cand_node.begin(), b.cand_node.begin() + b.n_cand, first) - b.cand_node.begin();
   }
   return st;
 }
@@ -1142,12 +1166,9 @@ echo::StagedPlan plan_staged(const GraphBuild &b, const Steps &st, int sigma, si
     while (((int64_t)1 << k) < x) ++k;
     return k;
   };
-  int64_t rows2 = 0, words2 = 0, segmax = 0, prow = 0, pword = 0, crows2 = 0, pcand = 0;
+  int64_t rows2 = 0, words2 = 0, segmax = 0, prow = 0, pword = 0;
   for (int64_t l = 0; l < st.L; ++l) {
     const int64_t r = b.seg_node_off[st.off[l + 1]] - b.seg_node_off[st.off[l]];
-    const int64_t nc = st.cand[l + 1] - st.cand[l];
-    crows2 = std::max(crows2, nc + pcand);
-    pcand = nc;
     rows2 = std::max(rows2, r + prow);
     words2 = std::max(words2, st.words[l] + pword);
     segmax = std::max(segmax, st.off[l + 1] - st.off[l]);
@@ -1155,26 +1176,17 @@ echo::StagedPlan plan_staged(const GraphBuild &b, const Steps &st, int sigma, si
     pword = st.words[l];
   }
   const int dmin = std::max(pow2(rows2), 4), rmin = std::max(pow2(words2), 4);
-  const int cring = std::max(pow2(crows2), 4);  // candidate ring: two levels' candidates
   const int vwant = std::min(std::max(pow2(4 * segmax), 6), 12);
   for (int d = dmin + 2; d >= dmin; --d)
     for (int v = vwant; v >= 6; --v)
       for (int r = rmin + 1; r >= rmin; --r) {
-        const size_t need = echo::staged_layout(sigma, v, (size_t)1 << d, r, (size_t)1 << cring).total;
-        if (need <= smem_cap && d < 31 && r < 31 && cring < 31) {
+        const size_t need = echo::staged_layout(sigma, v, (size_t)1 << d, r).total;
+        if (need <= smem_cap && d < 31 && r < 31) {
           best.ok = true;
           best.dring_log2 = d;
           best.vring_log2 = v;
           best.rring_log2 = r;
-          best.cring_log2 = cring;
           best.smem = need;
-          // the pipelined kernel's duration ring takes every row the rest leaves:
-          // more levels in flight hide more of each level's copy latency
-          const int64_t row = (int64_t)sigma * 8, fixed = (int64_t)echo::staged_layout(sigma, v, 0, r, 0).total;
-          const int64_t crows = std::max<int64_t>(crows2, 2), room = (int64_t)smem_cap - fixed;
-          best.pipe_crows = (uint32_t)crows;
-          best.pipe_drows = (uint32_t)std::max<int64_t>(room / row, (int64_t)1 << d);
-          best.pipe_drows_c = (uint32_t)std::max<int64_t>((room - crows * row) / row, (int64_t)1 << d);
           return best;
         }
       }
@@ -1199,7 +1211,6 @@ void build_records(const GraphBuild &b, const Steps &stp, int sigma, int vlog2, 
     meta[4 * l] = (uint32_t)base;
     meta[4 * l + 1] = (uint32_t)i0;
     meta[4 * l + 2] = (uint32_t)s0;
-    meta[4 * l + 3] = (uint32_t)stp.cand[l];
     recs.resize(base + 4 * (s1 - s0), 0);
     for (int64_t t = s0; t < s1; ++t) {
       const int64_t h = b.seg_node_off[t], z = b.seg_node_off[t + 1] - 1;
@@ -1222,21 +1233,6 @@ void build_records(const GraphBuild &b, const Steps &stp, int sigma, int vlog2, 
       }
       recs.insert(recs.end(), far.begin(), far.end());
       recs[hd + 1] = nin | ((uint32_t)far.size() << 16);
-      // chain nodes that are overlap candidates: a 64-bit mask over the chain and the
-      // level-order index of the first of them
-      uint64_t mask = 0;
-      int64_t c_first = -1;
-      for (int64_t v = h; v <= z; ++v)
-        if (b.cand_flag[v]) {
-          mask |= 1ull << (v - h);
-          if (c_first < 0) c_first = b.cidx[v];
-        }
-      if (mask) {
-        recs[hd + 3] |= 1u << 16;
-        recs.push_back((uint32_t)mask);
-        recs.push_back((uint32_t)(mask >> 32));
-        recs.push_back((uint32_t)c_first);
-      }
       // chain positions before the tail whose finish a later step reads
       uint64_t kmask = 0;
       for (int64_t v = h; v < z; ++v)
@@ -1252,8 +1248,233 @@ void build_records(const GraphBuild &b, const Steps &stp, int sigma, int vlog2, 
   meta[4 * stp.L] = (uint32_t)recs.size();
   meta[4 * stp.L + 1] = (uint32_t)b.V;
   meta[4 * stp.L + 2] = (uint32_t)b.n_seg;
-  meta[4 * stp.L + 3] = (uint32_t)stp.cand[stp.L];
   if (recs.empty()) recs.assign(4, 0);
+}
+
+// The levelled composer's plan for scenario blocks of `sigma` (echo_levels.cu): a
+// shared-memory slot for every segment tail that a later head reads, the steps, each
+// step's chunk of the ring with its records and row lists, and the head programs.
+struct LevelPlan {
+  bool ok = false;
+  int64_t L = 0;
+  uint32_t prog_bytes = 0, prog_at = 0, ring_at = 0, ring_bytes = 0, smem_bytes = 0;
+  int32_t head_warps = 1, sum_warps = 1, store_warps = 1, sum_team = 1, store_team = 1;
+  // one buffer of everything the device reads, and the words at which its parts start
+  // (the copies' descriptors at 0; ends: its size)
+  std::vector<uint32_t> words;
+  int64_t heads = 0, recs_all = 0, recs_kept = 0, ends = 0;
+};
+
+LevelPlan plan_levels(const GraphBuild &b, int sigma, size_t smem_cap) {
+  LevelPlan P;
+  if (!b.stageable || b.n_seg == 0) return P;
+  const int64_t row = (int64_t)sigma * 8, pad = sigma == 1 ? 1 : 0;
+  const bool walks = echo::level_walks(sigma);
+  auto r16 = [](int64_t x) { return (x + 15) & ~(int64_t)15; };
+  const int64_t val_bytes = r16(b.n_slots * row);
+  if ((size_t)val_bytes > smem_cap / 2) return P;
+  auto place_of_slot = [&](int64_t s) { return (uint32_t)((echo::kLvFixedBytes + s * row) / 8); };
+  // Head threads for nine tenths of the levels' segments, at most 128 segments and 8 warps
+  // (blocks of 4 scenarios and more: 5); the wider levels take several steps.  (GPT-175B,
+  // first composition: x 250, 4 / 6 warps 1157 / 1072 us; x 1024, where the instructions
+  // of all warps count, 3 / 5 / 8 warps 2400 / 2283 / 2479 us.)
+  const int64_t lanes_h = sigma >= 4 ? sigma / 2 : sigma;  // head threads of a segment
+  std::vector<int64_t> widths(b.Ls);
+  for (int64_t l = 0; l < b.Ls; ++l) widths[l] = b.seg_lvl_off[l + 1] - b.seg_lvl_off[l];
+  std::nth_element(widths.begin(), widths.begin() + (b.Ls - 1) * 9 / 10, widths.end());
+  const int64_t wide = std::min<int64_t>(widths[(b.Ls - 1) * 9 / 10], 128);
+  P.head_warps = (int32_t)std::min<int64_t>((wide * lanes_h + 31) / 32, sigma >= 4 ? 5 : 8);
+  const int64_t per_step = P.head_warps * 32 / lanes_h;
+  P.prog_bytes = (uint32_t)(16 * per_step);
+  auto more_pieces = [&](int64_t t) {  // 16-byte pieces of the list of segment t's inputs
+    const int64_t nin = b.hin_off[t + 1] - b.hin_off[t];
+    return nin <= 4 ? (int64_t)0 : nin <= 10 ? (int64_t)1 : 1 + (nin - 10 + 7) / 8;
+  };
+  // bytes of a step's parts, as its segments are added
+  struct Part {
+    int64_t segs = 0, rows = 0, kept = 0, cands = 0, more = 0;  // kept: entries of the kept rows' list; more: bytes of the lists of inputs
+  };
+  struct Chunk {
+    int64_t list, map, dur, cand, start, total;  // byte offsets
+  };
+  auto chunk = [&](const Part &p) {
+    Chunk c;
+    c.list = echo::kLvDescBytes + r16(4 * p.segs) + (p.cands ? 16 * p.segs : 0);
+    c.map = c.list + p.more;
+    c.dur = c.map + r16(walks ? 16 * p.kept : std::max(2 * p.rows, 4 * p.kept));
+    c.cand = c.dur + r16((p.rows + 2 * pad) * row);
+    c.start = c.cand + (p.cands ? r16((p.cands + 2 * pad) * row) : 0);
+    c.total = c.start + r16(p.segs * row);
+    return c;
+  };
+  auto add = [&](Part p, int64_t t) {
+    ++p.segs;
+    p.more += 16 * more_pieces(t);
+    p.rows += b.seg_node_off[t + 1] - b.seg_node_off[t];
+    p.cands += __builtin_popcountll(b.seg_cand[t]);
+    const int64_t kept = __builtin_popcountll(b.seg_keep[t]);
+    p.kept += walks ? kept > 0 : kept;
+    return p;
+  };
+  P.prog_at = (uint32_t)(echo::kLvFixedBytes + val_bytes);
+  P.ring_at = P.prog_at + echo::kLvStages * P.prog_bytes;
+  const int64_t ring = ((int64_t)smem_cap - P.ring_at - echo::kLvSlackBytes) & ~(int64_t)15;
+  if (ring <= 0) return P;
+  std::vector<int64_t> off;
+  std::vector<Part> parts;
+  std::vector<int64_t> place, dep;
+  bool fits = false;
+  // (x 1024: chunks of an eighth / a fifth / a quarter of the ring 2815 / 2204 / 2590 us)
+  for (int64_t limit = ring / (sigma >= 4 ? 5 : 8); !fits && limit >= 1024; limit -= limit / 8) {
+    off.assign(1, 0);
+    parts.clear();
+    for (int64_t l = 0; l < b.Ls; ++l) {
+      Part p;
+      for (int64_t t = b.seg_lvl_off[l]; t < b.seg_lvl_off[l + 1]; ++t) {
+        const Part q = add(p, t);
+        if (p.segs && (chunk(q).total > limit || q.segs > per_step || q.rows > kStepNodes)) {
+          off.push_back(t);
+          parts.push_back(p);
+          p = add(Part{}, t);
+        } else {
+          p = q;
+        }
+      }
+      off.push_back(b.seg_lvl_off[l + 1]);
+      parts.push_back(p);
+    }
+    // chunks in the ring, one after another (one that does not fit before the end starts
+    // over), and for each the newest one whose space it takes
+    const int64_t L = (int64_t)parts.size();
+    place.assign(L, 0);
+    dep.assign(L, -1);
+    fits = true;
+    int64_t pos = 0, oldest = 0;
+    for (int64_t l = 0; l < L && fits; ++l) {
+      const int64_t s = chunk(parts[l]).total;
+      if (pos + s > ring) pos = 0;
+      for (int64_t m = l - 1; m >= oldest; --m)
+        if (place[m] < pos + s && pos < place[m] + chunk(parts[m]).total) {
+          dep[l] = m;
+          oldest = m + 1;
+          break;
+        }
+      if (l > 0) dep[l] = std::max(dep[l], dep[l - 1]);
+      place[l] = pos;
+      pos += s;
+      // (two steps are resident together: one is copied while the other is composed)
+      fits = s <= ring && (dep[l] < 0 || dep[l] <= l - 2);
+    }
+  }
+  if (!fits) return P;
+  P.L = (int64_t)parts.size();
+  P.ring_bytes = (uint32_t)ring;
+  P.smem_bytes = (uint32_t)(P.ring_at + ring + echo::kLvSlackBytes);
+  const uint32_t zero = place_of_slot(0), nobody = place_of_slot(1);
+  const int64_t L4 = (P.L + echo::kLvGroup - 1) / echo::kLvGroup * echo::kLvGroup;
+  P.heads = P.L * 16;
+  P.recs_all = P.heads + L4 * (int64_t)P.prog_bytes / 4;
+  P.recs_kept = P.recs_all;
+  for (const Part &p : parts) P.recs_kept += (chunk(p).map + (walks ? 0 : r16(2 * p.rows))) / 4;
+  P.ends = P.recs_kept;
+  for (const Part &p : parts) P.ends += (chunk(p).map + r16((walks ? 16 : 4) * p.kept)) / 4;
+  P.words.assign((size_t)P.ends, 0);
+  uint16_t *const progs = reinterpret_cast<uint16_t *>(P.words.data() + P.heads);
+  const uint16_t blank[8] = {(uint16_t)zero, (uint16_t)nobody, (uint16_t)nobody, (uint16_t)zero,
+                             (uint16_t)zero, (uint16_t)zero,   (uint16_t)zero,   0};
+  for (int64_t k = 0; k < L4 * per_step; ++k) std::memcpy(progs + 8 * k, blank, sizeof blank);  // entries without a segment
+  uint32_t *rec = P.words.data() + P.recs_all, *rec_kept = P.words.data() + P.recs_kept;  // the step's records
+  for (int64_t l = 0; l < P.L; ++l) {
+    const Part &p = parts[l];
+    const Chunk c = chunk(p);
+    const int64_t s0 = off[l], s1 = off[l + 1], i0 = b.seg_node_off[s0];
+    const int64_t d0 = echo::kLvDescBytes / 4, recs = d0 * 4 + r16(4 * p.segs);  // words of the descriptor; byte offset of the masks
+    uint16_t *seg_of_row = reinterpret_cast<uint16_t *>(rec + c.map / 4);
+    uint32_t *kept = rec_kept + c.map / 4;
+    uint16_t *prog = progs + l * per_step * 8;
+    uint16_t *rec16 = reinterpret_cast<uint16_t *>(rec);
+    int64_t more = c.list, cand0 = -1;
+    for (int64_t t = s0; t < s1; ++t) {
+      const int64_t k = t - s0, v0 = b.seg_node_off[t], len = b.seg_node_off[t + 1] - v0;
+      const uint64_t mask = b.seg_cand[t], keep = b.seg_keep[t];
+      const int64_t c_first = mask ? b.cidx[v0 + __builtin_ctzll(mask)] : 0, last_kept = keep ? 64 - __builtin_clzll(keep) : 0;
+      if (!walks) {
+        std::fill(seg_of_row + (v0 - i0), seg_of_row + (v0 - i0 + len), (uint16_t)k);
+        for (uint64_t m = keep; m; m &= m - 1) *kept++ = (uint32_t)(v0 - i0 + __builtin_ctzll(m)) | ((uint32_t)k << 16);
+      }
+      if (walks && keep)
+        for (uint32_t x : {(uint32_t)k | ((uint32_t)last_kept << 16), 0u, (uint32_t)keep, (uint32_t)(keep >> 32)}) *kept++ = x;
+      if (mask && cand0 < 0) cand0 = c_first;  // (candidates are numbered in row order)
+      rec[d0 + k] = (uint32_t)(v0 - i0) | ((uint32_t)len << 16) | ((mask ? 1u : 0u) << 24);
+      if (mask) {
+        uint32_t *cw = rec + recs / 4 + 4 * k;
+        cw[0] = (uint32_t)mask;
+        cw[1] = (uint32_t)(mask >> 32);
+        cw[2] = (uint32_t)(c_first - cand0);
+      }
+      const int64_t nin = b.hin_off[t + 1] - b.hin_off[t];
+      auto in = [&](int64_t q) { return q < nin ? place_of_slot(b.seg_slot[b.seg_int[b.hin[b.hin_off[t] + q]]]) : zero; };
+      const int64_t dur_at = P.ring_at + place[l] + c.dur + (i0 & pad) * row;
+      uint16_t *h = prog + 8 * k;
+      h[1] = (uint16_t)((P.ring_at + place[l] + c.start + k * row) / 8);
+      h[0] = walks ? h[1] : (uint16_t)((dur_at + (v0 - i0 + len - 1) * row) / 8);  // (a start replaces its sum)
+      h[2] = (uint16_t)place_of_slot(b.seg_slot[t]);
+      for (int i = 0; i < 4; ++i) h[3 + i] = (uint16_t)in(i);
+      if (const int64_t n = more_pieces(t)) {
+        h[7] = (uint16_t)((P.ring_at + place[l] + more) / 8);
+        rec16[more / 2] = (uint16_t)n;
+        for (int64_t i = 2; i < 8 * n; ++i) rec16[more / 2 + i] = (uint16_t)in(4 + i - 2);
+        more += 16 * n;
+      }
+    }
+    cand0 = std::max<int64_t>(cand0, 0);
+    uint32_t *m = rec;
+    m[0] = (uint32_t)(place[l] + echo::kLvDescBytes);
+    m[1] = (uint32_t)p.segs | ((uint32_t)p.rows << 16);
+    m[2] = (uint32_t)(place[l] + c.dur + (i0 & pad) * row);
+    m[3] = (uint32_t)(place[l] + c.start);
+    m[4] = (uint32_t)p.kept | ((uint32_t)p.cands << 16);
+    m[5] = (uint32_t)i0;
+    m[6] = (uint32_t)(place[l] + c.cand + (cand0 & pad) * row);
+    m[7] = (uint32_t)(place[l] + c.map);
+    // the copies: rows of one scenario (8 bytes) take the 16-byte aligned range around them
+    const int64_t ra = i0 & ~pad, rb = (i0 + p.rows + pad) & ~pad;
+    const int64_t ca = cand0 & ~pad, cb = p.cands ? (cand0 + p.cands + pad) & ~pad : ca;
+    auto copy = [&](int which, int64_t at, int64_t src, int64_t n) {
+      uint32_t *q = P.words.data() + 4 * (which * P.L + l);
+      q[0] = (uint32_t)(place[l] + at);
+      q[1] = (uint32_t)(int32_t)dep[l];
+      q[2] = (uint32_t)src;
+      q[3] = (uint32_t)n;
+    };
+    const int64_t n_all = (c.map + (walks ? 0 : r16(2 * p.rows))) / 4, n_kept = (c.map + r16((walks ? 16 : 4) * p.kept)) / 4;
+    copy(0, 0, (rec - P.words.data() - P.recs_all) / 4, n_all / 4);
+    copy(1, 0, (rec_kept - P.words.data() - P.recs_kept) / 4, n_kept / 4);
+    copy(2, c.dur, ra, rb - ra);
+    copy(3, c.cand, ca, cb - ca);
+    std::memcpy(rec_kept, rec, (size_t)c.map);
+    rec += n_all;
+    rec_kept += n_kept;
+  }
+  // 8 warps to sum, the rest to store, in teams large enough that a warp has about two
+  // units of 32 segments to sum and eight of 32 vectors to store in a step.  The teams of a
+  // role divide the stages: a stage's previous step is then the same team's, whose wait by
+  // phase parity needs that step to be over.
+  const int64_t lanes = sigma >= 2 ? sigma / 2 : 1;  // threads of a row
+  auto team = [](int64_t units, int64_t each, int most) {
+    int t = 1;
+    while (t < most && t * each < units) t *= 2;
+    return t;
+  };
+  P.sum_warps = 8;
+  P.sum_team = team(b.n_seg * lanes / (32 * P.L), 2, 4);
+  P.store_team = team(b.V * lanes / (32 * P.L), 8, 8);
+  P.store_warps = P.store_team;
+  while (2 * P.store_warps <= echo::kLvMaxWarps - 1 - echo::kLvCopyWarps - P.head_warps - P.sum_warps &&
+         2 * P.store_warps / P.store_team <= echo::kLvStages)
+    P.store_warps *= 2;
+  P.ok = true;
+  return P;
 }
 
 // ------------------------------------------------------------------------------------
@@ -1312,16 +1533,17 @@ struct echo_ctx {
   size_t cd_elems = 0;                    // elements of each compact matrix
   int32_t *cand_cidx = nullptr, *cidx = nullptr, *cand_node = nullptr;
   uint8_t *ov = nullptr;
-  uint32_t *d_recs = nullptr, *d_meta = nullptr;
+  uint32_t *d_recs = nullptr, *d_meta = nullptr;  // staged kernel's records; its or the levelled composer's plan
   echo::StagedPlan plan;
-  Steps steps;  // composition steps of the staged kernels
+  Steps steps;  // composition steps of the staged kernel
+  LevelPlan lplan;  // plan of the levelled composer (its words are on the device, d_meta: empty here)
   uint32_t rec_words = 0;
   std::vector<double> h_sums, h_maxsf;
   int final_f = 0;
   const int64_t *final_cd = nullptr;  // candidates' durations of the last composition (null: the original)
   bool have_ov = false;
   echo::OverlapArgs last_ov{};  // inputs of the last validator pass (to recompute its decisions)
-  int kernel_choice = 0;            // 0 automatic, 1 direct, 2 staged, 3 pipelined, 4 dataflow (tuning and tests)
+  int kernel_choice = 0;            // 0 automatic, 1 direct, 2 staged, 3 levelled, 4 dataflow (tuning and tests)
   // dataflow composer
   bool use_df = false;
   int64_t *df_off = nullptr;
@@ -1746,13 +1968,13 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
     if ((rc = activate_fold(c, h_flag == 0))) return rc;
   }
   const int64_t V = B.V;
-  // The dataflow composer (rows of 32 scenarios, a warp per rank) is serial in
-  // the length of the longest rank program, the levelled ones in their number of
-  // steps.  Measured on GB300: a program entry costs about 0.22 us while at most
-  // 8 warps share an SM, and proportionally more beyond (0.24 us on GPT-1.3B x 256,
-  // 0.37 us at 13.5 warps per SM on the 1024-rank workload, 0.52 us at 20 on
-  // GPT-175B x 1024); a levelled step costs about 1.1 us.  The cheaper estimate
-  // wins (when every warp can be resident).
+  // The dataflow composer (rows of 32 scenarios, a warp per rank) is serial in the length
+  // of the longest rank program, the levelled one in its number of steps.  Measured on
+  // GB300: a program entry costs about 0.22 us while at most 8 warps share an SM, and
+  // proportionally more beyond; a levelled step about 0.22 us and 0.026 us per KB of its
+  // rows (GPT-1.3B x 1, 256: 0.24 and 0.29 us with 2 and 4 KB a step; GPT-175B x 250, 1024:
+  // 0.37 and 0.65 us with 6 and 17 KB).  The cheaper estimate wins (when every warp can be
+  // resident).
   const int32_t n_groups = (S + 31) / 32;
   bool use_df = false;
   if (B.df_ok && (c->kernel_choice == 0 || c->kernel_choice == 4) &&
@@ -1761,14 +1983,25 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
     for (int32_t r = 0; r < B.R; ++r) longest = std::max(longest, B.df_off[r + 1] - B.df_off[r]);
     const double warps_per_sm = (double)B.R * n_groups / std::max(c->sms, 1);
     const double df_us = (double)longest * 0.22 * std::max(1.0, warps_per_sm / 8.0);
-    const double lev_us = (double)make_steps(B, kStepNodes).L * 1.1;
+    // (steps of at most 128 segments or a fifth of the ring; rows of all blocks' scenarios)
+    const int lev_sigma = pick_sigma(S, c->sms);
+    double steps = 0;
+    for (int64_t l = 0; l < B.Ls; ++l) {
+      const int64_t segs = B.seg_lvl_off[l + 1] - B.seg_lvl_off[l];
+      const int64_t rows = B.seg_node_off[B.seg_lvl_off[l + 1]] - B.seg_node_off[B.seg_lvl_off[l]];
+      steps += (double)std::max<int64_t>({1, (segs + 127) / 128, rows * lev_sigma * 8 / 40000});
+    }
+    const double lev_us = steps * 0.22 + (double)B.V * lev_sigma * 8 / 1024 * 0.026;
     use_df = c->kernel_choice == 4 || df_us < lev_us;
   }
   const int sigma = use_df ? 32 : pick_sigma(S, c->sms);
   int slog2 = 0;
   while ((1 << slog2) < sigma) ++slog2;
   // [op][scenario] matrices are stored in scenario blocks of sigma (the last padded)
-  const size_t VS = (size_t)V * (size_t)((S + sigma - 1) / sigma) * sigma;
+  // (rows of one scenario start on 16-byte boundaries: an even number of them a block)
+  const int64_t pitch = sigma == 1 ? (V + 1) & ~(int64_t)1 : V;
+  const int64_t c_rows = std::max<int64_t>(B.n_cand, 1), c_pitch = sigma == 1 ? (c_rows + 1) & ~(int64_t)1 : c_rows;
+  const size_t VS = (size_t)pitch * (size_t)((S + sigma - 1) / sigma) * sigma;
   const int32_t G = (int32_t)B.sigs.size();
   if (c->scen_vs != VS || c->S != S || c->C != C || c->sigma != sigma || c->use_df != use_df) {
     free_all(c->scen_allocs);
@@ -1777,7 +2010,7 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
     bool in_smem = true;
     echo::compose_smem_bytes(B.R * B.NS, sigma, &in_smem);
     int64_t nblk = (S + sigma - 1) / sigma;
-    const size_t CS = (size_t)std::max<int64_t>(B.n_cand, 1) * (size_t)nblk * sigma;  // compact matrices
+    const size_t CS = (size_t)c_pitch * (size_t)nblk * sigma;  // compact matrices
     if ((rc = dalloc(c, o, &c->prm, (size_t)6 * S)) || (rc = dalloc(c, o, &c->sf, (size_t)C * S)) ||
         (rc = dalloc(c, o, &c->sums, (size_t)S)) || (rc = dalloc(c, o, &c->comm_sum, (size_t)S)) ||
         (rc = dalloc(c, o, &c->dur, VS)) ||
@@ -1818,38 +2051,43 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
     if (const char *e = std::getenv("ECHO_STAGED_THREADS")) threads = std::atoi(e);
     if (const char *e = std::getenv("ECHO_BLOCKS_PER_SM")) bps = std::max(1, std::atoi(e));
     const size_t cap = std::min((size_t)std::max(optin - 1024, 0), (size_t)(per_sm / bps) - 1024);
-    // the widest steps whose rings fit
-    for (int64_t step_cap = kStepNodes; !use_df; step_cap /= 2) {
+    c->lplan = LevelPlan{};
+    c->plan = echo::StagedPlan{};
+    if (!use_df && (c->kernel_choice == 0 || c->kernel_choice == 3)) {
+      LevelPlan &P = c->lplan;
+      P = plan_levels(B, sigma, (size_t)std::max(optin - 1024, 0));
+      if (P.ok) {
+        if ((rc = upload(c, o, &c->d_meta, P.words))) {
+          free_all(c->scen_allocs);
+          return rc;
+        }
+        CK(cudaStreamSynchronize(c->stream), "plan upload");
+        P.words = std::vector<uint32_t>();
+      }
+    }
+    // the staged kernel: the widest steps whose rings fit
+    for (int64_t step_cap = kStepNodes; !use_df && !c->lplan.ok && c->kernel_choice != 1; step_cap /= 2) {
       c->steps = make_steps(B, step_cap);
       c->plan = plan_staged(B, c->steps, sigma, cap);
       if (c->plan.ok || step_cap <= 2 * echo::kMaxSegment) break;
     }
-    if (use_df) c->plan = echo::StagedPlan{};
-    const Steps &st = c->steps;
     c->plan.threads = threads;
     if (c->plan.ok) {
-      // the pipelined kernel moves whole rows of even width and arms each step's
-      // byte count on one mbarrier (transaction counts stay below 2^20)
-      int64_t max_bytes = 0;
-      for (int64_t l = 0; l < st.L; ++l) {
-        const int64_t rows = B.seg_node_off[st.off[l + 1]] - B.seg_node_off[st.off[l]];
-        max_bytes = std::max(max_bytes, rows * sigma * 8 + st.words[l] * 4 + 32 + (st.cand[l + 1] - st.cand[l]) * sigma * 8);
-      }
-      c->plan.pipelined = sigma % 2 == 0 && max_bytes < (1 << 20);
       std::vector<uint32_t> recs, meta;
-      build_records(B, st, sigma, c->plan.vring_log2, recs, meta);
-      c->rec_words = meta[4 * st.L];
+      build_records(B, c->steps, sigma, c->plan.vring_log2, recs, meta);
+      c->rec_words = meta[4 * c->steps.L];
       if ((rc = upload(c, o, &c->d_recs, recs)) || (rc = upload(c, o, &c->d_meta, meta))) {
         free_all(c->scen_allocs);
         return rc;
       }
+      CK(cudaStreamSynchronize(c->stream), "record upload");
     }
     c->scen_vs = VS;
     c->S = S;
     c->C = C;
     c->sigma = sigma;
-    c->lay = echo::MatLayout{V, slog2};
-    c->lay_c = echo::MatLayout{B.n_cand, slog2};
+    c->lay = echo::MatLayout{pitch, slog2};
+    c->lay_c = echo::MatLayout{c_pitch, slog2};
     c->cd_elems = CS;
   }
   c->tbl = tbl;
@@ -1938,9 +2176,9 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
   const char *dbg_env = std::getenv("ECHO_DEBUG_BOUNDS");
   const int32_t dbg = (opts && opts->debug_bounds) || (dbg_env && std::atoi(dbg_env) != 0) ? 1 : 0;
   const GraphBuild &B = c->gb;
-  // the pipelined and dataflow kernels read the validator's durations of the
+  // the levelled and dataflow composers read the validator's durations of the
   // candidates (compact rows); the others compose from a full matrix built for them
-  const bool ring = c->use_df || (c->plan.ok && c->plan.pipelined && (c->kernel_choice == 0 || c->kernel_choice == 3));
+  const bool ring = c->use_df || c->lplan.ok;
   if (refine > 1 && !c->cd[1]) {
     if ((rc = dalloc(c, c->scen_allocs, &c->cd[1], c->cd_elems))) return rc;
     CK(cudaMemsetAsync(c->cd[1], 0, c->cd_elems * sizeof(int64_t), c->stream), "memset");
@@ -1988,8 +2226,8 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
     o.status = c->status;
     return o;
   };
-  // one composition with durations `d` (and, for the pipelined and dataflow
-  // kernels, the candidates' durations `cdur`) into `f`
+  // one composition with durations `d` (and, for the levelled and dataflow
+  // composers, the candidates' durations `cdur`) into `f`
   // (final_pass: the readback reads every finish of this composition)
   auto compose_pass = [&](const int64_t *d, const int64_t *cdur, int64_t *f, bool adjusted,
                           bool final_pass) -> cudaError_t {
@@ -2035,37 +2273,57 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
         return err;
       return timed(c, name, [&] { return echo::launch_compose_dataflow(a, c->stream); });
     }
+    if (c->lplan.ok) {
+      echo::LevelArgs a{};
+      a.S = c->S;
+      a.L = (int32_t)c->lplan.L;
+      a.pitch = c->lay.V;
+      a.c_pitch = c->lay_c.V;
+      a.meta = c->d_meta;
+      a.recs_all = c->d_meta + c->lplan.recs_all;
+      a.recs_kept = c->d_meta + c->lplan.recs_kept;
+      a.dur = d;
+      a.cdur = B.n_cand ? cdur : nullptr;
+      a.f = f;
+      a.makespan = c->mk;
+      a.heads = c->d_meta + c->lplan.heads;
+      a.prog_bytes = c->lplan.prog_bytes;
+      a.prog_at = c->lplan.prog_at;
+      a.ring_at = c->lplan.ring_at;
+      a.ring_bytes = c->lplan.ring_bytes;
+      a.smem_bytes = c->lplan.smem_bytes;
+      a.head_warps = c->lplan.head_warps;
+      a.sum_warps = c->lplan.sum_warps;
+      a.store_warps = c->lplan.store_warps;
+      a.sum_team = c->lplan.sum_team;
+      a.store_team = c->lplan.store_team;
+      a.status = c->status;
+      a.wait_limit_cycles = c->wait_limit_cycles;
+      a.skip_level = c->skip_level;
+      a.store_all = final_pass;
+      a.dbg = dbg;
+      a.n_recs_all = (c->lplan.recs_kept - c->lplan.recs_all) / 4;
+      a.n_recs_kept = (c->lplan.ends - c->lplan.recs_kept) / 4;
+      return timed(c, name, [&] { return echo::launch_compose_levels(a, c->sigma, c->stream); });
+    }
     if (c->plan.ok && c->kernel_choice != 1) {
       echo::StagedArgs a{};
       a.S = c->S;
       a.L = (int32_t)c->steps.L;
       a.n_rows = (uint32_t)B.V;
       a.n_words = c->rec_words;
+      a.pitch = c->lay.V;
       a.vlog2 = c->plan.vring_log2;
       a.dlog2 = c->plan.dring_log2;
       a.rlog2 = c->plan.rring_log2;
-      a.clog2 = c->plan.cring_log2;
-      a.d_rows = (uint32_t)1 << c->plan.dring_log2;
-      a.c_rows = (uint32_t)1 << c->plan.cring_log2;
       a.meta = c->d_meta;
       a.recs = c->d_recs;
       a.dur = d;
-      a.cdur = cdur;
-      a.n_cand = (uint32_t)B.n_cand;
       a.f = f;
       a.makespan = c->mk;
       a.status = c->status;
-      a.wait_limit_cycles = c->wait_limit_cycles;
-      a.skip_level = c->skip_level;
       a.store_all = final_pass;
       a.dbg = dbg;
-      const bool pipe = c->plan.pipelined && (c->kernel_choice == 0 || c->kernel_choice == 3);
-      if (pipe) {
-        a.d_rows = cdur ? c->plan.pipe_drows_c : c->plan.pipe_drows;
-        a.c_rows = cdur ? c->plan.pipe_crows : 0;
-      }
-      if (pipe)
-        return timed(c, name, [&] { return echo::launch_compose_pipelined(a, c->sigma, c->plan, c->stream); });
       return timed(c, name, [&] { return echo::launch_compose_staged(a, c->sigma, c->plan, c->stream); });
     }
     echo::ComposeArgs a{};
@@ -2340,11 +2598,11 @@ int echo_graph_info_get(echo_ctx *c, echo_graph_info *info) {
   info->n_overlap_candidates = B.cand_off.empty() ? 0 : B.cand_off.back();
   info->n_validator_comm_entries = B.cq_off.empty() ? 0 : B.cq_off.back();
   info->n_kept_finishes = B.V;
-  if (!c->use_df) {  // segment tails and the ops whose finish the validator reads
+  if (!c->use_df) {  // the ops whose finish the validator reads (and the segment tails, for the staged kernel)
     int64_t n = 0;
     for (int64_t t = 0; t < B.n_seg; ++t)
       for (int64_t v = B.seg_node_off[t]; v < B.seg_node_off[t + 1]; ++v)
-        n += (v + 1 == B.seg_node_off[t + 1]) || B.keep[v];
+        n += (!c->lplan.ok && v + 1 == B.seg_node_off[t + 1]) || B.keep[v];
     info->n_kept_finishes = n;
   }
   info->n_ranks = B.R;

@@ -20,8 +20,6 @@ constexpr int kOvBatch = 8;                // candidates per batch of the overla
 constexpr int kOvDepth = 3;                // batches of candidate rows in flight per warp
 constexpr int kOvWarps = 4;                // warps per block of the overlap test
 constexpr int kMaxSegment = 64;            // longest serial chain composed as one segment
-constexpr int kPipeStages = 16;            // stages (mbarrier pairs) of the pipelined compose
-constexpr int kPipeConsumerWarps = 16;     // composing warps of the pipelined compose
 
 // device status word: first error wins
 enum DeviceStatus : int32_t {
@@ -80,72 +78,113 @@ struct ComposeArgs {
   int32_t *status;
 };
 
-// Staged and pipelined compose: per-segment-level records and duration rows are
-// copied into shared-memory rings ahead of use.  Record block of a level (32-bit
-// words): for each segment, 4 header words {offset of its entries in the block,
-// nin | nfar << 16, first node - level's first node, length}; entries = the
-// head's nin inputs held in the value ring (byte offsets of their slots), then its
-// nfar inputs too old for the ring (node ids, read from global memory).  Every
-// input is the tail of an earlier segment.  A segment whose chain holds overlap
-// candidates has bit 16 of its length word set and 3 more entries: a 64-bit mask
-// of those chain positions and the level-order index of the first.  A segment with
-// chain positions before its tail whose finish a later step reads (validator
-// inputs) has bit 17 set and 2 more entries: the 64-bit mask of those positions.
-// Blocks are padded to 4 words.  Metadata of a level: record word offset, first node, first
-// segment, first level-order candidate.
+// Staged compose: per-segment-level records and duration rows are copied into
+// shared-memory rings ahead of use.  Record block of a level (32-bit words): for each
+// segment, 4 header words {offset of its entries in the block, nin | nfar << 16, first
+// node - level's first node, length}; entries = the head's nin inputs held in the
+// value ring (byte offsets of their slots), then its nfar inputs too old for the ring
+// (node ids, read from global memory).  Every input is the tail of an earlier segment.
+// A segment with chain positions before its tail whose finish a later step reads
+// (validator inputs) has bit 17 of its length word set and 2 more entries: the 64-bit
+// mask of those positions.  Blocks are padded to 4 words.  Metadata of a level: record
+// word offset, first node, first segment, 0.
 struct StagedArgs {
   int32_t S, L;                  // L: segment levels
   uint32_t n_rows, n_words;      // nodes; words of all record blocks
+  int64_t pitch;                 // rows of a scenario block of dur and f
   int32_t vlog2, dlog2, rlog2;   // log2 sizes: value ring (segments), duration ring (rows), record ring (words)
-  uint32_t d_rows, c_rows;       // ring sizes in rows (any size): duration and candidate rings
-  const uint32_t *meta;          // [4*(L+1)]: record word offset, first node, first segment, first candidate
+  const uint32_t *meta;          // [4*(L+1)]: record word offset, first node, first segment, 0
   const uint32_t *recs;          // record blocks
   const int64_t *dur;            // durations (MatLayout)
   int64_t *f;                    // finish times (MatLayout, out)
   int64_t *makespan;             // [S] (out)
-  // pipelined kernel only
-  const int64_t *cdur;           // validator durations of the candidates ([n_cand] rows per block), or null
-  uint32_t n_cand;               // overlap candidates
-  int32_t clog2;                 // log2 rows of the candidate ring (staged kernel)
-  int32_t *status;               // device status word (kDevTimeout when a bounded wait gives up)
-  long long wait_limit_cycles;   // bound of every mbarrier wait, in SM clock cycles
-  int32_t skip_level;            // failure injection for tests: this level is never filled (-1: none)
+  int32_t *status;               // device status word
   int32_t store_all;             // final composition: store every finish; else only those read again
   int32_t dbg;                   // debug bounds: check every index (echo_bounds.h)
 };
 
-// Plan of the staged kernels for one (graph, sigma); see plan_staged().
+// Plan of the staged kernel for one (graph, sigma); see plan_staged().
 struct StagedPlan {
   bool ok = false;
-  bool pipelined = false;  // bulk-copy producer warp (even sigma)
-  int threads = 512;       // threads per block of the staged kernel
+  int threads = 512;       // threads per block
   int vring_log2 = 0, dring_log2 = 0, rring_log2 = 0;  // sizes (segments, rows, words)
-  int cring_log2 = 0;  // candidate ring (rows of the validator's durations, pipelined kernel)
   size_t smem = 0;
-  // the pipelined kernel's rings take rows of any count, so they fill the shared
-  // memory left: without a candidate ring (a composition with the original
-  // durations) and with one (a composition that reads the validator's)
-  uint32_t pipe_drows = 0, pipe_drows_c = 0, pipe_crows = 0;
 };
 
-// Shared-memory layout of the staged kernels (byte offsets).  Every region starts
+// Shared-memory layout of the staged kernel (byte offsets).  Every region starts
 // on a 16-byte boundary, as 16-byte copy destinations require.
 struct StagedLayout {
-  size_t hist, meta, vr, dr, rr, cr, total;
+  size_t hist, meta, vr, dr, rr, total;
 };
 __host__ __device__ inline size_t round16(size_t x) { return (x + 15) & ~(size_t)15; }
-// d_rows, c_rows: rows of the duration and candidate rings.
-__host__ __device__ inline StagedLayout staged_layout(int sigma, int vlog2, size_t d_rows, int rlog2, size_t c_rows) {
+// d_rows: rows of the duration ring.
+__host__ __device__ inline StagedLayout staged_layout(int sigma, int vlog2, size_t d_rows, int rlog2) {
   StagedLayout L;
   L.hist = 128;                        // [0, 128): per-scenario makespans
   L.meta = L.hist + 16 * 8;            // 16 copy-group extents
   L.vr = L.meta + round16((size_t)2 * kMetaCap * 16);
   L.dr = L.vr + round16(((size_t)1 << vlog2) * sigma * 8);
   L.rr = L.dr + round16(d_rows * sigma * 8);
-  L.cr = L.rr + round16(((size_t)1 << rlog2) * 4);
-  L.total = L.cr + round16(c_rows * sigma * 8);
+  L.total = L.rr + round16(((size_t)1 << rlog2) * 4);
   return L;
 }
+
+// Levelled composer (echo_levels.cu).  The composition runs in steps (a segment
+// level or a part of one).  Shared memory: barriers and descriptors, the slots of the
+// tails' finishes (slot 0 holds 0, slot 1 takes what nobody reads), the head programs
+// of kLvStages steps, and the ring of chunks, one a step: records, row
+// list, duration rows (then their running sums), the candidates' rows, the segments'
+// starts.  The host places all of it (plan_levels).
+// Descriptor of a step: {byte offset in the ring of the records, segments | rows << 16,
+// byte offsets in the ring of the durations and of the starts; kept rows | candidates
+// << 16, first row, byte offsets in the ring of the candidates' durations and of the row
+// list}.  Records of a step: 4 bytes a segment {first row | length << 16 |
+// (candidates ? 1 : 0) << 24}; if the step holds candidates, 16 bytes a segment {mask of
+// their chain positions (64 bits), first row among the step's candidates, 0}; the row
+// list: for the final composition (recs_all) the 16-bit segment of every row of the step,
+// for the others (recs_kept) row | segment << 16 of every row that a later step reads.
+// Where the store warps walk segments (level_walks): no list, and 16 bytes a segment with
+// such rows {segment | rows up to its last one << 16, 0, mask of them (64 bits)}; "kept"
+// in the descriptor counts these.
+// The lists of inputs beyond four lie between the masks and the row list: 16-byte pieces,
+// the first {pieces, inputs 5-10}, the others 8 inputs each, 16 bits an input.
+// Head program of a step: 16 bytes for every segment the head threads can take
+// (echo_levels.cu, head_role); a step has no more segments than that.
+constexpr int kLvStages = 16;      // steps in flight (barriers of each); a power of two
+constexpr int kLvGroup = 4;        // steps of one copy of head programs
+constexpr int kLvMaxWarps = 32;    // of a block
+constexpr int kLvDescBytes = 32;   // step descriptor, at the start of its records
+constexpr int kLvCopyWarps = 4;    // divides kLvStages
+constexpr int kLvFixedBytes = 144 + 4 * kLvStages * 8 + kLvStages / kLvGroup * 8 + kLvStages * 12;
+// whether the store warps of blocks of `sigma` scenarios walk the segments (echo_levels.cu, sum_role)
+constexpr bool level_walks(int sigma) { return sigma >= 4; }
+constexpr int kLvSlackBytes = 1024;  // after the ring: loads past a segment's end
+
+struct LevelArgs {
+  int32_t S, L;                    // scenarios, steps
+  int64_t pitch, c_pitch;          // rows of a scenario block of dur / f, of cdur
+  // [4][L] copies of each step: records with all rows, with kept rows (16-byte units),
+  // durations, candidates' durations (rows): {byte offset in the ring, last step that
+  // must have been stored before (-1: none), first unit, units}
+  const uint32_t *meta;
+  const uint32_t *recs_all, *recs_kept;
+  const int64_t *dur;              // durations (MatLayout)
+  const int64_t *cdur;             // candidates' durations (compact), or null: the original ones
+  int64_t *f;                      // finish times (MatLayout, out)
+  int64_t *makespan;               // [S] (out)
+  const uint32_t *heads;           // head programs
+  uint32_t prog_bytes;             // of a step's head program
+  uint32_t prog_at, ring_at;       // byte offsets in shared memory of the head programs, of the ring
+  uint32_t ring_bytes, smem_bytes; // size of the ring, of all shared memory
+  int32_t head_warps, sum_warps, store_warps;
+  int32_t sum_team, store_team;    // warps that share a step; the number of teams of a role divides kLvStages
+  int32_t *status;
+  long long wait_limit_cycles;     // bound of every wait, in SM clock cycles
+  int32_t skip_level;              // failure injection for tests: this step is never filled (-1: none)
+  int32_t store_all;               // final composition: store every finish; else those a later step reads
+  int32_t dbg;                     // debug bounds: check every index (echo_bounds.h)
+  int64_t n_recs_all, n_recs_kept;  // its bounds: 16-byte units of the records
+};
 
 // Validator: for each overlap candidate (a compute op), whether its interval
 // overlaps a comm op of its rank, and the duration to use in the next composition.
@@ -257,7 +296,7 @@ cudaError_t launch_permute_rows(const void *raw, int bits, const int32_t *int2ex
                                 cudaStream_t st);
 cudaError_t launch_compose(const ComposeArgs &a, int sigma, cudaStream_t st);
 cudaError_t launch_compose_staged(const StagedArgs &a, int sigma, const StagedPlan &plan, cudaStream_t st);
-cudaError_t launch_compose_pipelined(const StagedArgs &a, int sigma, const StagedPlan &plan, cudaStream_t st);
+cudaError_t launch_compose_levels(const LevelArgs &a, int sigma, cudaStream_t st);
 cudaError_t launch_overlap(const OverlapArgs &a, cudaStream_t st);
 cudaError_t launch_readback(const int32_t *ext2int, int64_t op0, int64_t op1, int32_t s0, int32_t s1, MatLayout lay,
                             const int64_t *f, const int64_t *d, const int32_t *cidx, MatLayout lay_c,

@@ -1,0 +1,60 @@
+"""The levelled composer at the edges of its plan, against the oracle: chains of 1 to 130 ops (segments hold at most 64,
+warps take 4 and 8 rows at a time), joins of 1 to 150 inputs (4 in the head program, 6 in the first piece of a list, 8 in
+each further one; more than 128 segments a level take two steps), asynchronous collectives that make overlap candidates of
+the chains beside them, and full and partial scenario blocks of every width."""
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2412_12487_gb300 import Echo
+from paper_2412_12487_gb300 import workloads as W
+
+from . import smallgraphs as SG
+from .test_gpu_parity import assert_same, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _joins(ranks, lengths):
+    """Rounds of a chain on every rank and a join of all ranks; on stream 2 a collective of the round that only the last
+    op waits for."""
+    ops, queues, waits = [], {(r, k): [] for r in range(ranks) for k in range(3)}, []
+    everyone = list(range(ranks))
+    join = None
+    for i in range(len(lengths)):
+        tails = []
+        for r in everyone:
+            for n in range(lengths[(i + r) % len(lengths)]):
+                queues[(r, 0)].append(len(ops))
+                ops.append({"kind": W.KIND_COMPUTE, "kclass": r % 3, "preds": [join] if n == 0 and join is not None else []})
+            tails.append(len(ops) - 1)
+        for stream in (1, 2):
+            for r in everyone:
+                queues[(r, stream)].append(len(ops))
+            if stream == 1:
+                join = len(ops)
+            else:
+                waits.append(len(ops))
+            ops.append({"kind": W.KIND_COLL, "group": 0, "cc_type": W.CC_ALLREDUCE, "cc_algo": W.ALGO_AUTO,
+                        "cc_bytes": 1 << (10 + i), "preds": tails})
+    queues[(0, 0)].append(len(ops))
+    ops.append({"kind": W.KIND_COMPUTE, "kclass": 0, "preds": waits + [join]})
+    return SG.graph_from_lists(ranks, 3, ops, queues, [everyone], gpus_per_node=4)
+
+
+@pytest.mark.parametrize("sigma", [1, 2, 4, 8, 16])
+@pytest.mark.parametrize("ranks", [1, 4, 5, 10, 11, 19, 150])
+def test_chain_and_join_edges_bit_exact(sigma, ranks, monkeypatch):
+    monkeypatch.setenv("ECHO_COMPOSE_KERNEL", "pipelined")
+    monkeypatch.setenv("ECHO_SIGMA", str(sigma))
+    g = _joins(ranks, [1, 3, 4, 5, 7, 8, 9] + ([63, 64, 65, 130] if ranks < 100 else [12]))
+    rng = np.random.default_rng(100 * sigma + ranks)
+    with Echo(0) as e:
+        for S in (sigma, 2 * sigma + 1):
+            sc = SG.random_scenarios(rng, g, S, max_dur=20_000)
+            for refine, model, interval in ((0, 0, 0), (1, 0, 0), (2, 1, 1)):
+                got = run_gpu(g, sc, refine, ctx=e, overlap_model=model, comm_interval=interval)
+                assert got["info"]["sigma"] == sigma
+                want = oracle.compose(g, sc, refine_passes=refine, overlap_model=model, comm_interval=interval)
+                assert_same(got, want, g, refine)
