@@ -65,12 +65,12 @@ struct GraphBuild {
   std::vector<int32_t> sig_count, comm_node, comm_sig, node_sig;
   std::vector<int64_t> cand_off;      // [R+1] overlap candidates of each rank (compute ops, issue order)
   std::vector<int32_t> cand_ops;      // (internal ids)
+  std::vector<uint4> cand_rec;        // {internal id, level-order index, kernel class, 0} of each entry of cand_ops
+  int64_t most_cands = 0;             // of one rank
   std::vector<uint8_t> cand_flag;     // [V] 1 for an overlap candidate
   int64_t n_cand = 0;                 // overlap candidates
   std::vector<int32_t> cidx;          // [V] level-order index of a candidate (by internal id), -1 otherwise
-  std::vector<int32_t> cand_cidx;     // level-order index of each entry of cand_ops
   std::vector<int32_t> cand_node;     // internal id of each candidate, in level order
-  std::vector<uint8_t> cand_kcl;      // kernel class of each entry of cand_ops
   std::vector<uint8_t> q_rel;         // [queue entries] 1 for a comm op that can overlap a compute op
                                       // of the entry's rank in some scenario (see overlap_candidates)
   int32_t n_cq = 0;                   // comm timelines per rank in cq_off (max over ranks)
@@ -133,7 +133,6 @@ void overlap_candidates(GraphBuild &b) {
   b.cand_off.assign(R + 1, 0);
   b.cand_ops.clear();
   b.cand_flag.assign(V, 0);
-  b.cand_kcl.clear();
   b.q_rel.assign(std::max<int64_t>(b.q_off[(int64_t)R * NS], 1), 0);
   std::vector<int32_t> nodes, cpos, prv, nxt, anc, desc;
   std::vector<int64_t> cover;
@@ -192,11 +191,11 @@ void overlap_candidates(GraphBuild &b) {
       if (run > 0) {
         const int32_t v = b.q_ops_int[c0 + p];
         b.cand_ops.push_back(v);
-        b.cand_kcl.push_back(b.kcl[v]);
         b.cand_flag[v] = 1;
       }
     }
     b.cand_off[r + 1] = (int64_t)b.cand_ops.size();
+    b.most_cands = std::max(b.most_cands, b.cand_off[r + 1] - b.cand_off[r]);
     for (int64_t j = 0; j < m; ++j) loc[nodes[j]] = -1;
   }
   // level order of the candidates (by internal id): each segment level's candidates
@@ -210,11 +209,11 @@ void overlap_candidates(GraphBuild &b) {
       b.cand_node.push_back((int32_t)v);
     }
   if (b.cand_node.empty()) b.cand_node.push_back(0);
-  b.cand_cidx.resize(b.cand_ops.size());
-  for (size_t k = 0; k < b.cand_ops.size(); ++k) b.cand_cidx[k] = b.n_cand ? b.cidx[b.cand_ops[k]] : 0;
-  if (b.cand_ops.empty()) b.cand_ops.push_back(0);
-  if (b.cand_kcl.empty()) b.cand_kcl.push_back(0);
-  if (b.cand_cidx.empty()) b.cand_cidx.push_back(0);
+  b.cand_rec.resize(std::max<size_t>(b.cand_ops.size(), 1));
+  for (size_t k = 0; k < b.cand_ops.size(); ++k) {
+    const int32_t v = b.cand_ops[k];
+    b.cand_rec[k] = make_uint4((uint32_t)v, (uint32_t)b.cidx[v], b.kcl[v], 0);
+  }
 }
 
 
@@ -1507,10 +1506,9 @@ struct echo_ctx {
   // device graph
   int64_t *seg_lvl_off = nullptr, *seg_node_off = nullptr, *nq_off = nullptr, *dp_off = nullptr, *q_off = nullptr;
   int64_t *cq_off = nullptr;
-  uint8_t *cand_kcl = nullptr;
+  uint4 *cand_rec = nullptr;
   int32_t *cq_ops = nullptr, *lq_off = nullptr, *lq_ops = nullptr;
   int64_t *cand_off = nullptr;
-  int32_t *cand_ops = nullptr;
   uint8_t *cand_flag = nullptr;
   int32_t *nq = nullptr, *dp = nullptr, *q_ops = nullptr, *int2ext = nullptr, *ext2int = nullptr;
   int32_t *node_sig = nullptr, *comm_node = nullptr, *comm_sig = nullptr, *sig_count = nullptr;
@@ -1531,7 +1529,7 @@ struct echo_ctx {
   int64_t *cd[2] = {nullptr, nullptr};    // candidates' durations of the validator's passes (compact)
   echo::MatLayout lay_c{0, 0};            // [n_cand][S] compact layout
   size_t cd_elems = 0;                    // elements of each compact matrix
-  int32_t *cand_cidx = nullptr, *cidx = nullptr, *cand_node = nullptr;
+  int32_t *cidx = nullptr, *cand_node = nullptr;
   uint8_t *ov = nullptr;
   uint32_t *d_recs = nullptr, *d_meta = nullptr;  // staged kernel's records; its or the levelled composer's plan
   echo::StagedPlan plan;
@@ -1712,11 +1710,11 @@ int upload_graph(echo_ctx *c) {
   auto &o = c->graph_allocs;
   int rc;
   if ((rc = upload(c, o, &c->seg_lvl_off, B.seg_lvl_off)) || (rc = upload(c, o, &c->seg_node_off, B.seg_node_off)) ||
-      (rc = upload(c, o, &c->cand_kcl, B.cand_kcl)) ||
+      (rc = upload(c, o, &c->cand_rec, B.cand_rec)) ||
       (rc = upload(c, o, &c->cq_off, B.cq_off)) || (rc = upload(c, o, &c->cq_ops, B.cq_ops)) ||
       (rc = upload(c, o, &c->lq_off, B.lq_off)) || (rc = upload(c, o, &c->lq_ops, B.lq_ops)) ||
-      (rc = upload(c, o, &c->cand_off, B.cand_off)) || (rc = upload(c, o, &c->cand_ops, B.cand_ops)) ||
-      (rc = upload(c, o, &c->cand_flag, B.cand_flag)) || (rc = upload(c, o, &c->cand_cidx, B.cand_cidx)) ||
+      (rc = upload(c, o, &c->cand_off, B.cand_off)) ||
+      (rc = upload(c, o, &c->cand_flag, B.cand_flag)) ||
       (rc = upload(c, o, &c->cidx, B.cidx)) || (rc = upload(c, o, &c->cand_node, B.cand_node)) ||
       (rc = upload(c, o, &c->nq_off, B.nq_off)) ||
       (rc = upload(c, o, &c->nq, B.nq)) || (rc = upload(c, o, &c->dp_off, B.dp_off)) ||
@@ -2196,18 +2194,16 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
     o.S = c->S;
     o.n_streams = B.NS;
     o.n_ranks = B.R;
-    {  // pieces of each rank's list: enough warps for about sixteen waves (16 warps
-       // per SM; shorter pieces even out the last wave: 9.27 -> 8.79 ms on the
-       // 1024-rank workload, 1.24 -> 1.09 ms on GPT-175B against four waves), each
-       // piece at least 64 candidates long
-      const int64_t base = (int64_t)B.R * ((c->S + 31) / 32), want = 16 * 16 * (int64_t)c->sms;
-      const int64_t per_rank = B.n_cand / std::max<int32_t>(B.R, 1);
-      o.parts = (int32_t)std::max<int64_t>(1, std::min((want + base - 1) / base, per_rank / 64));
+    o.rows = B.V;
+    o.c_rows = B.n_cand;
+    {  // pieces of each rank's list: enough warps for about eight waves (24 warps an SM; the
+       // pieces are not all of one length), each at least four batches of candidates long
+      const int64_t base = (int64_t)B.R * ((c->S + c->sigma - 1) / c->sigma), want = 8 * 24 * (int64_t)c->sms;
+      const int64_t batch = (int64_t)echo::kOvBatch * (32 / c->sigma);
+      o.parts = (int32_t)std::max<int64_t>(1, std::min((want + base - 1) / base, B.most_cands / (4 * batch)));
     }
-    o.cand_kcl = c->cand_kcl;
+    o.cand_rec = c->cand_rec;
     o.cand_off = c->cand_off;
-    o.cand_ops = c->cand_ops;
-    o.cand_cidx = c->cand_cidx;
     o.n_cq = B.n_cq;
     o.cq_off = c->cq_off;
     o.cq_ops = c->cq_ops;

@@ -16,9 +16,11 @@ constexpr int kComposeThreads = 512;       // direct compose kernel
 constexpr int kMetaChunk = 128;            // segment levels of metadata staged at a time
 constexpr int kMetaCap = 136;              // metadata entries per staging buffer (>= kMetaChunk + 1)
 constexpr uint32_t kFarRef = 0x80000000u;  // predecessor reference read from global memory
-constexpr int kOvBatch = 8;                // candidates per batch of the overlap test
-constexpr int kOvDepth = 3;                // batches of candidate rows in flight per warp
+constexpr int kOvBatch = 4;                // candidates a lane tests between two waits (overlap test)
 constexpr int kOvWarps = 4;                // warps per block of the overlap test
+// shared memory of a warp of it: records of three batches (16 bytes for every team),
+// finish, duration and factor of two batches
+__host__ __device__ constexpr size_t overlap_warp_bytes(int teams) { return 3 * kOvBatch * 16 * teams + 2 * kOvBatch * 3 * 256; }
 constexpr int kMaxSegment = 64;            // longest serial chain composed as one segment
 
 // device status word: first error wins
@@ -195,9 +197,9 @@ struct OverlapArgs {
   int32_t n_cq;            // comm timelines per rank (lists of a rank with fewer are empty)
   int32_t n_ranks;
   int32_t parts;           // pieces of each rank's candidate list (one warp per piece and 32 scenarios)
-  const int64_t *cand_off; const int32_t *cand_ops;  // [R+1]: each rank's overlap candidates, in issue order
-  const int32_t *cand_cidx;                          // level-order index of each entry of cand_ops
-  const uint8_t *cand_kcl;                           // kernel class of each entry of cand_ops
+  int64_t rows, c_rows;    // of the matrices, of the compact ones
+  const int64_t *cand_off; const uint4 *cand_rec;  // [R+1]: each rank's overlap candidates, in issue order: {node,
+                                                   // level-order index, kernel class, 0}
   const int64_t *cq_off; const int32_t *cq_ops;  // [R*n_cq+1]: comm ops of each (rank, comm timeline)
   // launch conditions of each entry of cq_ops on its rank (CSR); null: a comm op's
   // interval is its execution [start, finish), else [latest of them, finish)
@@ -265,9 +267,6 @@ cudaError_t launch_compose_dataflow(const DataflowArgs &a, cudaStream_t st);
 size_t dataflow_smem_bytes(int32_t n_streams, int32_t wpb);
 // whether every warp of R * G warps can be resident at once (cooperative launch)
 bool dataflow_fits(int64_t n_warps, int32_t n_streams, int32_t wpb, int device);
-
-// shared memory of an overlap-test block: each warp's ring of candidate rows
-inline size_t overlap_smem_bytes() { return (size_t)kOvWarps * kOvDepth * kOvBatch * 2 * 32 * sizeof(int64_t); }
 
 // overlap.cu: the overlap test, one entry point per (launch interval, proportional
 // model) pair, each dispatching on the number of comm timelines

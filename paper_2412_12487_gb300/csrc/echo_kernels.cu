@@ -234,25 +234,6 @@ __global__ void __launch_bounds__(256, 6) permute_rows_kernel(const T *__restric
 }
 
 // ---------------------------------------------------------------------------------
-// B3: validator overlap test over the overlap candidates: the compute ops that
-// some comm op of their rank is neither an ancestor nor a descendant of (the
-// others can never overlap; their durations are copied unchanged).  One thread
-// per (chunk of a rank's candidates, which run in issue order, scenario); a warp
-// covers 32 scenarios of one chunk and shares its op list.
-// Every timeline of a rank runs its ops one after the other, so on each of the
-// rank's comm timelines the intervals are sorted and the compute ops' starts only
-// grow.  The thread keeps, per comm timeline, a cursor at the first comm op of
-// positive length that finishes after the current candidate starts, with that
-// op's interval in registers: the compute op overlaps this timeline iff that
-// interval starts before the compute op finishes (any later comm op starts after
-// the cursor op ends).  A binary search places the cursors at the chunk's first
-// op; from there they only move forward, and only then touch memory.  A compute
-// op of positive length that overlaps gets rint(d * slowdown) for the next
-// composition (cd_next, compact), others keep d; the decisions themselves are stored only
-// when `ov` is given.  The finish times and durations of 8 consecutive ops are
-// loaded together before they are tested.
-// ---------------------------------------------------------------------------------
-// ---------------------------------------------------------------------------------
 // readback: internal order and blocked layout -> caller order, [op][scenario]
 // ---------------------------------------------------------------------------------
 // start = finish - the duration the op had in the last composition: d, or for an
@@ -472,9 +453,9 @@ cudaError_t launch_replica_check(const void *raw, int bits, const int32_t *pairs
 }
 
 cudaError_t launch_overlap(const OverlapArgs &a, cudaStream_t st) {
-  const int64_t warps = (int64_t)a.n_ranks * ((a.S + 31) / 32) * a.parts;
+  const int64_t warps = (int64_t)a.n_ranks * ((a.S + (1 << a.lay.slog2) - 1) >> a.lay.slog2) * a.parts;
   if (a.S == 0 || warps == 0) return cudaSuccess;
-  if (a.n_cq < 0 || a.n_cq > kMaxStreams || a.parts < 1) return cudaErrorInvalidValue;
+  if (a.n_cq < 0 || a.n_cq > kMaxStreams || a.parts < 1 || a.lay.slog2 > 5) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)((warps + kOvWarps - 1) / kOvWarps));
   const int tx = kOvWarps * 32;
   // the variants are compiled in four translation units (echo_overlap.cu)
