@@ -21,7 +21,21 @@ namespace {
 constexpr int kAR = 0, kAG = 1, kSR = 3;  // reduce-scatter (2) takes the generic ring path
 constexpr int kRing = 0, kTree = 1;
 
-__device__ __forceinline__ int64_t cdiv64(int64_t a, int64_t b) { return (a + b - 1) / b; }
+// ceil(a / b), a >= 0, b > 0.  Quotients of the estimator (chunk rounds) are small, and a
+// 64-bit division takes about 100 instructions: an estimate in fp32 is off by at most
+// q * 2^-21 + 1 < 2 below 2^20, which the remainder puts right.
+__device__ __forceinline__ int64_t cdiv64(int64_t a, int64_t b) {
+  const int64_t n = a + b - 1;
+  const float q0 = __fdividef((float)n, (float)b);
+  if (!(q0 < 1048576.0f) || n < 0 || b >= (1ll << 40)) return n / b;
+  int32_t q = (int32_t)q0;
+  int64_t r = n - (int64_t)q * b;
+  if (r < 0) { --q; r += b; }
+  if (r < 0) { --q; r += b; }
+  if (r >= b) { ++q; r -= b; }
+  if (r >= b) ++q;
+  return q;
+}
 
 __device__ __forceinline__ int64_t chunk_for(int64_t nbytes, const ChunkTable &t) {
   for (int i = 0; i < t.n; ++i)
@@ -29,35 +43,54 @@ __device__ __forceinline__ int64_t chunk_for(int64_t nbytes, const ChunkTable &t
   return t.chunk[t.n - 1];
 }
 
+// x as a double, 0 <= x, rounded to nearest even: below 2^53 the bits are put together in
+// integers, as a conversion occupies the fp64 pipe (527 G operations/s on this part, a
+// seventieth of its integer rate) like an addition.
+__device__ __forceinline__ double to_double(int64_t x) {
+  if ((uint64_t)x >> 53) return (double)x;
+  const int up = __clzll(x) - 11;  // puts the highest bit at bit 52
+  const uint64_t bits = (((uint64_t)x << (up & 63)) & ((1ull << 52) - 1)) | ((uint64_t)(1075 - up) << 52);
+  return __longlong_as_double(x ? (int64_t)bits : 0);
+}
+// The product of two such doubles: exact in integers when it stays below 2^53.
+__device__ __forceinline__ double product(int64_t x, int64_t y) {
+  if (((uint64_t)x | (uint64_t)y) >> 31 || (x * y) >> 53) return __dmul_rn(to_double(x), to_double(y));
+  return to_double(x * y);
+}
+
 // Eqs. 2-4 (Sec. 5.3): eta chunk rounds, eta*(N-1) ring steps (twice that for
-// all-reduce), each L + p/B with p = S/(N*eta); inter-node link once M > 1.
-__device__ double ring_ns(int type, int64_t S, int N, int M, double alpha, double Ba, double La,
-                          double Be, double Le, double delta, int64_t C) {
-  int64_t eta = cdiv64(S, (int64_t)N * C);
+// all-reduce), each L + p/B with p = S/(N*eta); inter-node link once M > 1.  Send/recv takes
+// the same operations: eta chunk transfers of S/eta over the pair's link.  One code path
+// for all of them, so that a warp of mixed queries runs it once.
+__device__ __forceinline__ double linear_ns(int type, int64_t S, int N, int M, double alpha, double Ba, double La,
+                                            double Be, double Le, double delta, int64_t C) {
+  const bool pair = type == kSR;
+  int64_t eta = cdiv64(S, pair ? C : (int64_t)N * C);
   if (eta < 1) eta = 1;
-  double p = __ddiv_rn((double)S, __dmul_rn((double)N, (double)eta));
-  double L = M > 1 ? Le : La;
-  double B = M > 1 ? Be : Ba;
-  double t = __dadd_rn(L, __ddiv_rn(p, B));
-  int64_t steps = (type == kAR ? 2 : 1) * eta * (int64_t)(N - 1);
-  double T = __dadd_rn(alpha, __dmul_rn((double)steps, t));
-  if (type != kAG) T = __dadd_rn(T, __dmul_rn(delta, (double)S));
-  return T;
+  const double size = to_double(S);
+  const double p = __ddiv_rn(size, pair ? to_double(eta) : product(N, eta));
+  const double L = M > 1 ? Le : La;
+  const double B = M > 1 ? Be : Ba;
+  const double t = __dadd_rn(L, __ddiv_rn(p, B));
+  const int64_t steps = pair ? eta : (type == kAR ? 2 : 1) * eta * (int64_t)(N - 1);
+  const double T = __dadd_rn(alpha, __dmul_rn(to_double(steps), t));
+  return type == kAG || pair ? T : __dadd_rn(T, __dmul_rn(delta, size));
 }
 
 // Eq. 5 (Sec. 5.3): tree all-reduce; eta chunks, K-1 intra-node hops (beta) and
 // log2(M) inter-node levels (gamma) up and down.
-__device__ double tree_ns(int64_t S, int M, int K, double lg, double alpha, double Ba, double La,
-                          double Be, double Le, double delta, int64_t C) {
+__device__ __forceinline__ double tree_ns(int64_t S, int M, int K, double lg, double alpha, double Ba, double La,
+                                          double Be, double Le, double delta, int64_t C) {
   int64_t eta = cdiv64(S, C);
   if (eta < 1) eta = 1;
-  double pt = __ddiv_rn((double)S, (double)eta);
+  const double size = to_double(S);
+  double pt = __ddiv_rn(size, to_double(eta));
   double beta = __dadd_rn(La, __ddiv_rn(pt, Ba));
   double gamma = M > 1 ? __dadd_rn(Le, __ddiv_rn(pt, Be)) : beta;
-  double T = __dadd_rn(alpha, __dmul_rn(gamma, (double)(eta - 1)));
-  T = __dadd_rn(T, __dmul_rn(__dmul_rn(2.0, beta), (double)(K - 1)));
+  double T = __dadd_rn(alpha, __dmul_rn(gamma, to_double(eta - 1)));
+  T = __dadd_rn(T, __dmul_rn(__dmul_rn(2.0, beta), to_double(K - 1)));
   T = __dadd_rn(T, __dmul_rn(__dmul_rn(2.0, gamma), lg));
-  T = __dadd_rn(T, __dmul_rn(delta, (double)S));
+  T = __dadd_rn(T, __dmul_rn(delta, size));
   return T;
 }
 
@@ -66,19 +99,10 @@ __device__ double cc_ns_of(int type, int algo, int64_t S, int N, int M, int K, d
                            const ChunkTable &tbl) {
   if (N <= 1 || S <= 0) return 0.0;
   int64_t C = chunk_for(S, tbl);
-  if (type == kSR) {  // send/recv: eta chunk transfers over the pair's link
-    int64_t eta = cdiv64(S, C);
-    if (eta < 1) eta = 1;
-    double L = M > 1 ? Le : La;
-    double B = M > 1 ? Be : Ba;
-    double per = __dadd_rn(L, __ddiv_rn(__ddiv_rn((double)S, (double)eta), B));
-    return __dadd_rn(alpha, __dmul_rn((double)eta, per));
-  }
-  if (type != kAR || algo == kRing) return ring_ns(type, S, N, M, alpha, Ba, La, Be, Le, delta, C);
-  if (algo == kTree) return tree_ns(S, M, K, lg, alpha, Ba, La, Be, Le, delta, C);
-  double r = ring_ns(kAR, S, N, M, alpha, Ba, La, Be, Le, delta, C);
-  double t = tree_ns(S, M, K, lg, alpha, Ba, La, Be, Le, delta, C);
-  return t < r ? t : r;
+  const bool ring = type != kAR || algo != kTree, tree = type == kAR && algo != kRing;
+  const double r = ring ? linear_ns(type, S, N, M, alpha, Ba, La, Be, Le, delta, C) : 0.0;
+  const double t = tree ? tree_ns(S, M, K, lg, alpha, Ba, La, Be, Le, delta, C) : 0.0;
+  return !tree ? r : !ring || t < r ? t : r;
 }
 
 __device__ __forceinline__ void set_status(int32_t *status, int32_t code) {
@@ -132,17 +156,70 @@ __global__ void cc_scatter_kernel(const int32_t *__restrict__ comm_node, const i
   }
 }
 
-__global__ void cc_query_kernel(int64_t n, const uint8_t *__restrict__ type, const uint8_t *__restrict__ algo,
-                                const int64_t *__restrict__ nbytes, const int32_t *__restrict__ N,
-                                const int32_t *__restrict__ M, const double *__restrict__ lg, ScenParams p,
-                                ChunkTable tbl, double *__restrict__ out) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int n_r = N[i], m = M[i];
-    int K = (n_r + m - 1) / m;
-    out[i] = cc_ns_of(type[i], algo[i], nbytes[i], n_r, m, K, lg[i], p.alpha[i], p.bwa[i], p.lata[i],
-                      p.bwe[i], p.late[i], p.delta[i], tbl);
+// A block's queries.  Every thread takes one as far as it is linear (send/recv and rings),
+// then the trees (a sixth of a mixed sweep) are gathered, so that two warps and not eight
+// run their code.  What bounds it is the fp64 pipe (divisions run at 73 G/s on this part):
+// two or three divisions a query.  With a branch per form, every warp of a mixed sweep ran
+// them all, some twelve divisions (a call with 10^6 queries on the device: 297 us, now 105;
+// with the fields loaded where they are used, one after the other, 205).
+// A query's inputs are read before its own result is written, and by no other thread
+// after that, so the output may be one of the input arrays.
+constexpr int kQueryThreads = 256;
+struct QueryShared {
+  int32_t n;                    // trees
+  uint16_t who[kQueryThreads];  // their threads
+  double ring[kQueryThreads];   // by thread: a ring's time that a tree's is to be compared with
+};
+struct Queries {
+  const uint8_t *type, *algo;
+  const int64_t *nbytes;
+  const int32_t *N, *M;
+  const double *lg;  // log2(M): by query, or by M
+  bool lg_by_m;
+  ScenParams p;
+};
+__device__ __forceinline__ void query_block(int64_t i, bool mine, const Queries &q, const ChunkTable &tbl, double *out,
+                                            QueryShared &sh) {
+  if (threadIdx.x == 0) sh.n = 0;
+  __syncthreads();
+  if (mine) {
+    // (all fields are asked for before the first is looked at)
+    const int type = q.type[i], algo = q.algo[i], N = q.N[i], M = q.M[i];
+    const int64_t S = q.nbytes[i];
+    const double alpha = q.p.alpha[i], bwa = q.p.bwa[i], lata = q.p.lata[i], bwe = q.p.bwe[i], late = q.p.late[i],
+                 delta = q.p.delta[i];
+    const bool some = N > 1 && S > 0;
+    const bool tree = some && type == kAR && algo != kRing;
+    double T = 0.0;
+    if (some && !(tree && algo == kTree))
+      T = linear_ns(type, S, N, M, alpha, bwa, lata, bwe, late, delta, chunk_for(S, tbl));
+    if (tree) {
+      sh.ring[threadIdx.x] = T;
+      sh.who[atomicAdd(&sh.n, 1)] = (uint16_t)threadIdx.x;
+    } else {
+      out[i] = T;
+    }
   }
+  __syncthreads();
+  if ((int)threadIdx.x < sh.n) {
+    const int w = sh.who[threadIdx.x];
+    const int64_t k = i - threadIdx.x + w;
+    const int algo = q.algo[k], N = q.N[k], M = q.M[k];
+    const int64_t S = q.nbytes[k];
+    const double alpha = q.p.alpha[k], bwa = q.p.bwa[k], lata = q.p.lata[k], bwe = q.p.bwe[k], late = q.p.late[k],
+                 delta = q.p.delta[k];
+    const double t = tree_ns(S, M, (N + M - 1) / M, q.lg[q.lg_by_m ? M : k], alpha, bwa, lata, bwe, late, delta,
+                             chunk_for(S, tbl));
+    const double r = sh.ring[w];
+    out[k] = algo == kTree || t < r ? t : r;
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kQueryThreads) cc_query_kernel(int64_t n, Queries q, ChunkTable tbl, double *out) {
+  __shared__ QueryShared sh;
+  for (int64_t i0 = (int64_t)blockIdx.x * kQueryThreads; i0 < n; i0 += (int64_t)gridDim.x * kQueryThreads)
+    query_block(i0 + threadIdx.x, i0 + threadIdx.x < n, q, tbl, out, sh);
 }
 
 // ---------------------------------------------------------------------------------
@@ -404,7 +481,7 @@ cudaError_t launch_cc_query(int64_t n, const uint8_t *type, const uint8_t *algo,
                             const int32_t *N, const int32_t *M, const double *lg, ScenParams p,
                             const ChunkTable &tbl, double *out, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  cc_query_kernel<<<grid_for(n, 256), 256, 0, st>>>(n, type, algo, nbytes, N, M, lg, p, tbl, out);
+  cc_query_kernel<<<grid_for(n, kQueryThreads), kQueryThreads, 0, st>>>(n, Queries{type, algo, nbytes, N, M, lg, false, p}, tbl, out);
   return cudaGetLastError();
 }
 
@@ -633,40 +710,38 @@ void noalloc_setup(NoallocDevice &d) {
   d.ptr = base;
 }
 
-__device__ __forceinline__ bool nonneg_finite(double x) { return isfinite(x) && x >= 0.0; }
+// (by their bits: a comparison of doubles occupies the fp64 pipe)
+__device__ __forceinline__ bool nonneg_finite(double x) {
+  const uint64_t u = (uint64_t)__double_as_longlong(x);
+  return (u >> 52 & 0x7ff) != 0x7ff && (!(u >> 63) || !(u << 1));
+}
+__device__ __forceinline__ bool pos_finite(double x) {
+  const uint64_t u = (uint64_t)__double_as_longlong(x);
+  return (u >> 52) < 0x7ff && u != 0;
+}
 
 // Same estimate as cc_query_kernel; log2(M) comes from the table in the static
 // array and each query is checked on the device, since its fields live there.
-__global__ void cc_query_noalloc_kernel(int64_t n, const uint8_t *__restrict__ type,
-                                        const uint8_t *__restrict__ algo, const int64_t *__restrict__ nbytes,
-                                        const int32_t *__restrict__ N, const int32_t *__restrict__ M,
-                                        ScenParams p, ChunkTable tbl, unsigned char *scratch,
-                                        double *__restrict__ out) {
-  int32_t *status = reinterpret_cast<int32_t *>(scratch);
-  const double *lg = reinterpret_cast<const double *>(scratch + kNoallocLgOffset);
+__global__ void __launch_bounds__(kQueryThreads) cc_query_noalloc_kernel(int64_t n, Queries q, ChunkTable tbl,
+                                                                         int32_t *status, double *out) {
+  __shared__ QueryShared sh;
+  const ScenParams &p = q.p;
   const double nan = __longlong_as_double(0x7ff8000000000000LL);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int t = type[i], a = algo[i];
-    const int n_r = N[i], m = M[i];
-    const int64_t nb = nbytes[i];
-    const bool ok = t <= kSR && (t != kAR || a <= 2) && nb >= 0 && n_r >= 1 && m >= 1 && m <= n_r &&
-                    nonneg_finite(p.alpha[i]) && nonneg_finite(p.lata[i]) && nonneg_finite(p.late[i]) &&
-                    nonneg_finite(p.delta[i]) && isfinite(p.bwa[i]) && p.bwa[i] > 0.0 &&
-                    isfinite(p.bwe[i]) && p.bwe[i] > 0.0;
-    if (!ok) {
-      out[i] = nan;
-      atomicOr(status, kNoallocBadQuery);
-      continue;
+  for (int64_t i0 = (int64_t)blockIdx.x * kQueryThreads; i0 < n; i0 += (int64_t)gridDim.x * kQueryThreads) {
+    const int64_t i = i0 + threadIdx.x;
+    bool mine = i < n;
+    if (mine) {
+      const int t = q.type[i], a = q.algo[i], n_r = q.N[i], m = q.M[i];
+      const bool ok = (t <= kSR) & ((t != kAR) | (a <= 2)) & (q.nbytes[i] >= 0) & (n_r >= 1) & (m >= 1) & (m <= n_r) &
+                      nonneg_finite(p.alpha[i]) & nonneg_finite(p.lata[i]) & nonneg_finite(p.late[i]) &
+                      nonneg_finite(p.delta[i]) & pos_finite(p.bwa[i]) & pos_finite(p.bwe[i]);
+      if (!ok || m > kNoallocMaxNodes) {
+        out[i] = nan;
+        atomicOr(status, ok ? kNoallocTooManyNodes : kNoallocBadQuery);
+        mine = false;
+      }
     }
-    if (m > kNoallocMaxNodes) {
-      out[i] = nan;
-      atomicOr(status, kNoallocTooManyNodes);
-      continue;
-    }
-    const int K = (n_r + m - 1) / m;
-    out[i] = cc_ns_of(t, a, nb, n_r, m, K, lg[m], p.alpha[i], p.bwa[i], p.lata[i], p.bwe[i], p.late[i],
-                      p.delta[i], tbl);
+    query_block(i, mine, q, tbl, out, sh);
   }
 }
 
@@ -710,8 +785,10 @@ extern "C" int echo_cc_query_noalloc(const echo_cc_query_desc *q, double *out_ns
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   if (cudaMemsetAsync(d.ptr, 0, sizeof(int32_t), st) != cudaSuccess) return ECHO_E_CUDA;
   ScenParams p{q->alpha_ns, q->bw_intra, q->lat_intra, q->bw_inter, q->lat_inter, q->delta};
-  cc_query_noalloc_kernel<<<grid_for(q->n, 256), 256, 0, st>>>(q->n, q->cc_type, q->cc_algo, q->nbytes,
-                                                                q->n_ranks, q->n_nodes, p, tbl, d.ptr, out_ns);
+  const Queries dq{q->cc_type, q->cc_algo, q->nbytes, q->n_ranks, q->n_nodes,
+                   reinterpret_cast<const double *>(d.ptr + kNoallocLgOffset), true, p};
+  cc_query_noalloc_kernel<<<grid_for(q->n, kQueryThreads), kQueryThreads, 0, st>>>(
+      q->n, dq, tbl, reinterpret_cast<int32_t *>(d.ptr), out_ns);
   if (cudaGetLastError() != cudaSuccess) return ECHO_E_CUDA;
   int32_t status = 0;
   if (cudaMemcpyAsync(&status, d.ptr, sizeof(int32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
