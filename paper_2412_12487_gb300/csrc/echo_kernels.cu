@@ -501,31 +501,58 @@ cudaError_t launch_permute_rows(const void *raw, int bits, const int32_t *int2ex
   return cudaGetLastError();
 }
 
-template <typename T>
-__global__ void replica_check_kernel(const T *__restrict__ raw, const int32_t *__restrict__ pairs, int64_t n_pairs,
-                                     int32_t S, int32_t *flag) {
-  const int64_t total = n_pairs * S;
-  bool diff = false;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = idx / S, s = idx - p * S;
-    diff |= raw[(int64_t)pairs[2 * p] * S + s] != raw[(int64_t)pairs[2 * p + 1] * S + s];
+// Are the rows of a replica and of its representative equal?  One stream over all rows;
+// HBM bounds it, so a row is compared in the widest words that its length and start allow
+// (16 bytes, else the durations' own), by a team of lanes with eight loads in flight each.
+// 143491 pairs of 500 durations of 32 bits: 308 us element by element with a 64-bit
+// division each, 61 us now.
+__device__ __forceinline__ uint32_t differ(uint32_t a, uint32_t b) { return a ^ b; }
+__device__ __forceinline__ uint32_t differ(uint64_t a, uint64_t b) { return a != b; }
+__device__ __forceinline__ uint32_t differ(uint4 a, uint4 b) {
+  return (a.x ^ b.x) | (a.y ^ b.y) | (a.z ^ b.z) | (a.w ^ b.w);
+}
+template <typename U>
+__global__ void replica_check_kernel(const U *__restrict__ raw, const int2 *__restrict__ pairs, int64_t n_pairs,
+                                     int32_t n, int32_t team_log2, int32_t *flag) {
+  const int32_t team = 1 << team_log2, lane = threadIdx.x & (team - 1);
+  uint32_t diff = 0;
+  for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> team_log2; p < n_pairs;
+       p += ((int64_t)gridDim.x * blockDim.x) >> team_log2) {
+    const int2 pr = __ldg(pairs + p);
+    const U *a = raw + (int64_t)pr.x * n, *b = raw + (int64_t)pr.y * n;
+    for (int32_t i = lane; i < n; i += 4 * team) {
+      U x[4], y[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (i + k * team < n) x[k] = __ldg(a + i + k * team), y[k] = __ldg(b + i + k * team);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (i + k * team < n) diff |= differ(x[k], y[k]);
+    }
   }
-  if (__any_sync(0xffffffffu, diff) && (threadIdx.x & 31) == 0) *flag = 1;
+  if (__any_sync(0xffffffffu, diff != 0) && (threadIdx.x & 31) == 0) *flag = 1;
+}
+template <typename U>
+void replica_check_rows(const void *raw, const int32_t *pairs, int64_t n_pairs, int64_t row_bytes, int32_t *flag,
+                        cudaStream_t st) {
+  const int32_t n = (int32_t)(row_bytes / (int64_t)sizeof(U));
+  int32_t team_log2 = 0;  // a lane takes four words of a row at a time
+  while (team_log2 < 5 && (4 << team_log2) < n) ++team_log2;
+  const int64_t blocks = std::min<int64_t>(((n_pairs << team_log2) + 255) / 256, 152 * 8);
+  replica_check_kernel<U><<<(unsigned)blocks, 256, 0, st>>>(
+      static_cast<const U *>(raw), reinterpret_cast<const int2 *>(pairs), n_pairs, n, team_log2, flag);
 }
 
 cudaError_t launch_replica_check(const void *raw, int bits, const int32_t *pairs, int64_t n_pairs, int32_t S,
                                  int32_t *flag, cudaStream_t st) {
   if (n_pairs == 0 || S == 0) return cudaSuccess;
-  const int64_t total = n_pairs * S;
-  const int threads = 256;
-  const int64_t blocks = std::min<int64_t>((total + threads - 1) / threads, 152 * 16);
-  if (bits == 32)
-    replica_check_kernel<int32_t><<<(unsigned)blocks, threads, 0, st>>>(static_cast<const int32_t *>(raw), pairs,
-                                                                         n_pairs, S, flag);
+  const int64_t row_bytes = (int64_t)S * (bits / 8);
+  if (row_bytes % 16 == 0)
+    replica_check_rows<uint4>(raw, pairs, n_pairs, row_bytes, flag, st);
+  else if (bits == 64)
+    replica_check_rows<uint64_t>(raw, pairs, n_pairs, row_bytes, flag, st);
   else
-    replica_check_kernel<int64_t><<<(unsigned)blocks, threads, 0, st>>>(static_cast<const int64_t *>(raw), pairs,
-                                                                         n_pairs, S, flag);
+    replica_check_rows<uint32_t>(raw, pairs, n_pairs, row_bytes, flag, st);
   return cudaGetLastError();
 }
 
