@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <array>
+#include <cfloat>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1514,6 +1515,11 @@ struct echo_ctx {
   int32_t *node_sig = nullptr, *comm_node = nullptr, *comm_sig = nullptr, *sig_count = nullptr;
   uint8_t *kcl = nullptr, *local = nullptr;
   CcSig *sigs = nullptr;
+  // [S] sums, [S] comm_sum, a status word, [S] makespans lie one behind the other in
+  // `small`, so that each call reads its status and results back with one copy
+  int64_t *small = nullptr;
+  std::vector<int64_t> h_small;
+  bool reads_host = false;  // kernels may read the caller's host arrays in place (a coherent link to its memory)
   int32_t *status = nullptr;
   // scenarios
   int32_t S = 0, C = 0, sigma = 1;
@@ -1662,17 +1668,36 @@ int pick_sigma(int32_t S, int sms) {
   return s;
 }
 
-int sync_status(echo_ctx *c, int32_t *host_status) {
-  CK(cudaMemcpyAsync(host_status, c->status, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream), "status readback");
-  CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+// Waits for the stream's work and reads words [first, end) of `small` into h_small;
+// *status gets the status word, which is one of them.
+int read_small(echo_ctx *c, int64_t first, int64_t end, int32_t *status) {
+  const cudaError_t copied = cudaMemcpyAsync(c->h_small.data() + first, c->small + first,
+                                             (size_t)(end - first) * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream);
+  CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");  // (whatever the copy said: kernels may be reading host arrays)
+  CK(copied, "status and result readback");
+  *status = (int32_t)(uint32_t)(uint64_t)c->h_small[2 * (size_t)c->S];
   return ECHO_OK;
 }
+
+// Are all of x finite and >= 0 (positive: > 0)?  (no branch an element, so that it is vectorised)
+bool all_finite(const double *x, int64_t n, bool positive) {
+  int64_t bad = 0;
+  if (positive)
+    for (int64_t i = 0; i < n; ++i) bad |= !((x[i] > 0.0) & (x[i] <= DBL_MAX));
+  else
+    for (int64_t i = 0; i < n; ++i) bad |= !((x[i] >= 0.0) & (x[i] <= DBL_MAX));
+  return !bad;
+}
+
 
 int check_params(echo_ctx *c, int64_t n, const double *alpha, const double *bwa, const double *lata,
                  const double *bwe, const double *late, const double *delta) {
   if (n > 0 && (!alpha || !bwa || !lata || !bwe || !late || !delta))
     return set_err(c, ECHO_E_INVALID_ARG, "link parameter arrays are required");
-  for (int64_t s = 0; s < n; ++s) {
+  if (all_finite(alpha, n, false) && all_finite(bwa, n, true) && all_finite(lata, n, false) && all_finite(bwe, n, true) &&
+      all_finite(late, n, false) && all_finite(delta, n, false))
+    return ECHO_OK;
+  for (int64_t s = 0; s < n; ++s) {  // which one
     if (!finite_nonneg(alpha[s]) || !finite_nonneg(lata[s]) || !finite_nonneg(late[s]) || !finite_nonneg(delta[s]))
       return set_err(c, ECHO_E_INVALID_ARG, "alpha, latencies and delta must be finite and >= 0 (entry " + std::to_string(s) + ")");
     if (!(std::isfinite(bwa[s]) && bwa[s] > 0.0) || !(std::isfinite(bwe[s]) && bwe[s] > 0.0))
@@ -1801,13 +1826,8 @@ int echo_create(echo_ctx **out, int device, void *cuda_stream) {
     }
     c->own_stream = true;
   }
-  void *st = nullptr;
-  if (cudaMalloc(&st, sizeof(int32_t)) != cudaSuccess) {
-    if (c->own_stream) cudaStreamDestroy(c->stream);
-    delete c;
-    return ECHO_E_OOM;
-  }
-  c->status = static_cast<int32_t *>(st);
+  int pageable = 0;
+  c->reads_host = cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, device) == cudaSuccess && pageable;
   if (const char *e = std::getenv("ECHO_COMPOSE_KERNEL")) {  // tuning and tests: force a compose kernel
     const std::string k(e);
     c->kernel_choice = k == "direct" ? 1 : k == "staged" ? 2 : k == "pipelined" ? 3 : k == "dataflow" ? 4 : 0;
@@ -1832,7 +1852,6 @@ int echo_destroy(echo_ctx *c) {
   free_all(c->fold_allocs);
   free_all(c->raw_allocs);
   if (c->stage) cudaFree(c->stage);
-  if (c->status) cudaFree(c->status);
   for (auto &r : c->recs) {
     cudaEventDestroy(r.second.first);
     cudaEventDestroy(r.second.second);
@@ -2010,16 +2029,21 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
     int64_t nblk = (S + sigma - 1) / sigma;
     const size_t CS = (size_t)c_pitch * (size_t)nblk * sigma;  // compact matrices
     if ((rc = dalloc(c, o, &c->prm, (size_t)6 * S)) || (rc = dalloc(c, o, &c->sf, (size_t)C * S)) ||
-        (rc = dalloc(c, o, &c->sums, (size_t)S)) || (rc = dalloc(c, o, &c->comm_sum, (size_t)S)) ||
+        (rc = dalloc(c, o, &c->small, (size_t)3 * S + 1)) ||
         (rc = dalloc(c, o, &c->dur, VS)) ||
         (rc = dalloc(c, o, &c->f[0], VS)) || (rc = dalloc(c, o, &c->f[1], VS)) ||
         (rc = dalloc(c, o, &c->cd[0], CS)) || (rc = dalloc(c, o, &c->ov, VS)) ||
-        (rc = dalloc(c, o, &c->mk, (size_t)S)) || (rc = dalloc(c, o, &c->cc_ns, (size_t)G * S)) ||
+        (rc = dalloc(c, o, &c->cc_ns, (size_t)G * S)) ||
         (rc = dalloc(c, o, &c->cc_dur, (size_t)G * S)) ||
         (!in_smem && (rc = dalloc(c, o, &c->gfrontier, (size_t)nblk * B.R * B.NS * sigma)))) {
       free_all(c->scen_allocs);
       return rc;
     }
+    c->sums = reinterpret_cast<double *>(c->small);
+    c->comm_sum = c->sums + S;
+    c->status = reinterpret_cast<int32_t *>(c->small + 2 * (size_t)S);
+    c->mk = c->small + 2 * (size_t)S + 1;
+    c->h_small.assign((size_t)3 * S + 1, 0);
     if (in_smem) c->gfrontier = nullptr;
     c->use_df = use_df;
     if (use_df) {
@@ -2092,22 +2116,27 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
   c->h_maxsf = maxsf;
   // parameters
   const double *src[6] = {sc->alpha_ns, sc->bw_intra, sc->lat_intra, sc->bw_inter, sc->lat_inter, sc->delta};
-  for (int k = 0; k < 6; ++k)
-    CK(cudaMemcpyAsync(c->prm + (size_t)k * S, src[k], S * sizeof(double), cudaMemcpyHostToDevice, c->stream), "parameter upload");
-  CK(cudaMemcpyAsync(c->sf, sc->slowdown, (size_t)C * S * sizeof(double), cudaMemcpyHostToDevice, c->stream),
-     "slowdown upload");
-  CK(cudaMemsetAsync(c->sums, 0, S * sizeof(double), c->stream), "memset");
-  CK(cudaMemsetAsync(c->status, 0, sizeof(int32_t), c->stream), "memset");
+  if (!c->reads_host) {
+    for (int k = 0; k < 6; ++k)
+      CK(cudaMemcpyAsync(c->prm + (size_t)k * S, src[k], S * sizeof(double), cudaMemcpyHostToDevice, c->stream), "parameter upload");
+    CK(cudaMemcpyAsync(c->sf, sc->slowdown, (size_t)C * S * sizeof(double), cudaMemcpyHostToDevice, c->stream),
+       "slowdown upload");
+  }
+  CK(cudaMemsetAsync(c->small, 0, (2 * (size_t)S + 1) * sizeof(int64_t), c->stream), "memset");
   if (V > 0) {
     CK(timed(c, "permute_rows", [&] {
          return echo::launch_permute_rows(c->raw, bits, c->int2ext, c->local, V, S, c->lay, c->dur, c->sums,
                                           c->status, c->stream);
        }), "permute_rows launch");
   }
-  c->h_sums.assign(S, 0.0);
-  CK(cudaMemcpyAsync(c->h_sums.data(), c->sums, S * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "sum readback");
+  // (one launch that reads the caller's arrays, and from here on no way out before the wait)
+  const cudaError_t loaded =
+      c->reads_host ? echo::launch_load_params(src, sc->slowdown, S, C, c->prm, c->sf, c->stream) : cudaSuccess;
   int32_t st = 0;
-  if ((rc = sync_status(c, &st))) return rc;
+  if ((rc = read_small(c, 0, 2 * (int64_t)S + 1, &st))) return rc;
+  CK(loaded, "parameter upload");
+  c->h_sums.resize(S);
+  std::memcpy(c->h_sums.data(), c->h_small.data(), S * sizeof(double));
   if (st == echo::kDevNegativeDuration) return set_err(c, ECHO_E_INVALID_ARG, "negative duration in dur");
   c->state = 2;
   return ECHO_OK;
@@ -2121,8 +2150,7 @@ static int run_estimate(echo_ctx *c, int policy) {
   c->state = 2;
   echo::ScenParams p{c->prm, c->prm + S, c->prm + 2 * (size_t)S, c->prm + 3 * (size_t)S,
                      c->prm + 4 * (size_t)S, c->prm + 5 * (size_t)S};
-  CK(cudaMemsetAsync(c->status, 0, sizeof(int32_t), c->stream), "memset");
-  CK(cudaMemsetAsync(c->comm_sum, 0, S * sizeof(double), c->stream), "memset");
+  CK(cudaMemsetAsync(c->comm_sum, 0, ((size_t)S + 1) * sizeof(int64_t), c->stream), "memset");  // (and the status)
   CK(timed(c, "cc_estimate", [&] {
        return echo::launch_cc_estimate(c->sigs, G, p, S, c->tbl, c->sig_count, c->cc_ns, c->cc_dur,
                                        c->comm_sum, c->status, c->cc_model, policy, c->stream);
@@ -2131,11 +2159,11 @@ static int run_estimate(echo_ctx *c, int policy) {
        return echo::launch_cc_scatter(c->comm_node, c->comm_sig, (int64_t)B.comm_node.size(), c->cc_dur, S,
                                       c->lay, c->dur, c->stream);
      }), "cc_scatter launch");
-  std::vector<double> comm(S, 0.0);
-  CK(cudaMemcpyAsync(comm.data(), c->comm_sum, S * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "readback");
   int32_t st = 0;
   int rc;
-  if ((rc = sync_status(c, &st))) return rc;
+  if ((rc = read_small(c, S, 2 * (int64_t)S + 1, &st))) return rc;
+  std::vector<double> comm(S);
+  std::memcpy(comm.data(), c->h_small.data() + S, S * sizeof(double));
   if (st == echo::kDevCcOverflow) return set_err(c, ECHO_E_OVERFLOW, "a collective's estimated time is not below 2^61 ns");
   // every finish time is at most the sum of all (slowed) durations of its scenario
   for (int32_t s = 0; s < S; ++s) {
@@ -2370,9 +2398,10 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
 }
 
 // Device-side failures of the last composition (a bounded wait that gave up).
-static int composition_status(echo_ctx *c) {
+// makespans: they come with the status, into h_small.
+static int composition_status(echo_ctx *c, bool makespans = false) {
   int32_t st = 0;
-  int rc = sync_status(c, &st);
+  int rc = read_small(c, 2 * (int64_t)c->S, (makespans ? 3 : 2) * (int64_t)c->S + 1, &st);
   if (rc) return rc;
   if (st == echo::kDevTimeout) {
     if (c->use_df) {  // words a warp never wrote must not carry a later launch's tag
@@ -2393,6 +2422,16 @@ static int composition_status(echo_ctx *c) {
   }
   if (st == echo::kDevBounds) return set_err(c, ECHO_E_BOUNDS, "a debug-bounds index check failed on the device");
   return ECHO_OK;
+}
+
+// Memory that the host reads and writes itself.
+static bool host_memory(const void *p) {
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeUnregistered || at.type == cudaMemoryTypeHost;
 }
 
 // NULL, or plain memory of the context's device.
@@ -2458,8 +2497,12 @@ int echo_read_makespan(echo_ctx *c, int64_t *out) {
   if (rc) return rc;
   if (!out) return set_err(c, ECHO_E_INVALID_ARG, "output is NULL");
   if (c->state < 4) return set_err(c, ECHO_E_STATE, "compose first");
-  if ((rc = composition_status(c))) return rc;
-  CK(cudaMemcpyAsync(out, c->mk, c->S * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream), "D2H");
+  if ((rc = composition_status(c, true))) return rc;
+  const void *mk = c->h_small.data() + 2 * (size_t)c->S + 1;
+  if (host_memory(out))
+    std::memcpy(out, mk, c->S * sizeof(int64_t));
+  else  // (a device buffer)
+    CK(cudaMemcpyAsync(out, c->mk, c->S * sizeof(int64_t), cudaMemcpyDefault, c->stream), "makespan readback");
   CK(cudaStreamSynchronize(c->stream), "makespan readback");
   return ECHO_OK;
 }
@@ -2531,37 +2574,60 @@ int echo_cc_query(echo_ctx *c, const echo_cc_query_desc *q, double *out_ns) {
   if ((rc = check_params(c, n, q->alpha_ns, q->bw_intra, q->lat_intra, q->bw_inter, q->lat_inter, q->delta))) return rc;
   ChunkTable tbl;
   if ((rc = make_table(c, q->n_chunk, q->chunk_max_bytes, q->chunk_bytes, &tbl))) return rc;
-  std::vector<double> lg(n);
-  std::vector<double> lg_cache(4097, -1.0);
+  // log2(M): a table by M, or one a query where groups span more nodes than that
+  constexpr int32_t kMaxTable = 4096;
+  int64_t bad = 0;
+  int32_t max_m = 0;
+  for (int64_t i = 0; i < n; ++i)
+    bad |= (q->cc_type[i] > ECHO_CC_SENDRECV) | ((q->cc_type[i] == ECHO_CC_ALLREDUCE) & (q->cc_algo[i] > ECHO_ALGO_AUTO));
+  for (int64_t i = 0; i < n; ++i) bad |= q->nbytes[i] < 0;
   for (int64_t i = 0; i < n; ++i) {
+    const int32_t m = q->n_nodes[i];
+    bad |= (q->n_ranks[i] < 1) | (m < 1) | (m > q->n_ranks[i]);
+    max_m = std::max(max_m, m);
+  }
+  for (int64_t i = 0; bad && i < n; ++i) {  // which one
     if (q->cc_type[i] > ECHO_CC_SENDRECV || (q->cc_type[i] == ECHO_CC_ALLREDUCE && q->cc_algo[i] > ECHO_ALGO_AUTO))
       return set_err(c, ECHO_E_INVALID_ARG, "query " + std::to_string(i) + ": bad type or algorithm");
     if (q->nbytes[i] < 0 || q->n_ranks[i] < 1 || q->n_nodes[i] < 1 || q->n_nodes[i] > q->n_ranks[i])
       return set_err(c, ECHO_E_INVALID_ARG, "query " + std::to_string(i) + ": need bytes >= 0 and 1 <= M <= N");
-    int32_t m = q->n_nodes[i];
-    if (m <= 4096) {
-      if (lg_cache[m] < 0) lg_cache[m] = std::log2((double)m);
-      lg[i] = lg_cache[m];
-    } else {
-      lg[i] = std::log2((double)m);
-    }
   }
-  // one staging allocation holds every query array: 6 param doubles, lg, bytes, N, M, type, algo, out
-  const size_t per = 6 * 8 + 8 + 8 + 4 + 4 + 1 + 1 + 8;
-  if ((rc = stage_reserve(c, per * (size_t)n + 256))) return rc;
+  const bool by_m = max_m <= kMaxTable;
+  std::vector<double> lg(by_m ? (size_t)max_m + 1 : (size_t)n, 0.0);
+  for (size_t i = by_m ? 1 : 0; i < lg.size(); ++i) lg[i] = std::log2((double)(by_m ? (int32_t)i : q->n_nodes[i]));
+  const double *src[6] = {q->alpha_ns, q->bw_intra, q->lat_intra, q->bw_inter, q->lat_inter, q->delta};
+  if (c->reads_host) {
+    // The kernel reads the caller's arrays where they are: of the 290 us that 20011 queries
+    // took, the twelve uploads were 105 (9 each, one after the other), the checks 100
+    // (with a branch a field), the kernel 11.
+    if ((rc = stage_reserve(c, (size_t)n * sizeof(double)))) return rc;
+    double *dout = static_cast<double *>(c->stage);
+    const echo::ScenParams p{src[0], src[1], src[2], src[3], src[4], src[5]};
+    cudaError_t e = timed(c, "cc_query", [&] {
+      return echo::launch_cc_query(n, q->cc_type, q->cc_algo, q->nbytes, q->n_ranks, q->n_nodes, lg.data(), by_m, p, tbl, dout,
+                                   c->stream);
+    });
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out_ns, dout, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+    const cudaError_t done = cudaStreamSynchronize(c->stream);  // (the arrays are the caller's again, whatever went wrong)
+    CK(e, "cc_query launch");
+    CK(done, "cc_query");
+    return ECHO_OK;
+  }
+  // one staging allocation holds every query array: 6 param doubles, bytes, out, lg, N, M, type, algo
+  const size_t per = 6 * 8 + 8 + 8 + 4 + 4 + 1 + 1;
+  if ((rc = stage_reserve(c, per * (size_t)n + lg.size() * 8 + 256))) return rc;
   char *base = static_cast<char *>(c->stage);
   double *dprm = reinterpret_cast<double *>(base);
-  double *dlg = dprm + 6 * n;
-  int64_t *dbytes = reinterpret_cast<int64_t *>(dlg + n);
+  int64_t *dbytes = reinterpret_cast<int64_t *>(dprm + 6 * n);
   double *dout = reinterpret_cast<double *>(dbytes + n);
-  int32_t *dN = reinterpret_cast<int32_t *>(dout + n);
+  double *dlg = dout + n;
+  int32_t *dN = reinterpret_cast<int32_t *>(dlg + lg.size());
   int32_t *dM = dN + n;
   uint8_t *dtype = reinterpret_cast<uint8_t *>(dM + n);
   uint8_t *dalgo = dtype + n;
-  const double *src[6] = {q->alpha_ns, q->bw_intra, q->lat_intra, q->bw_inter, q->lat_inter, q->delta};
   for (int k = 0; k < 6; ++k)
     CK(cudaMemcpyAsync(dprm + (size_t)k * n, src[k], n * sizeof(double), cudaMemcpyHostToDevice, c->stream), "H2D");
-  CK(cudaMemcpyAsync(dlg, lg.data(), n * sizeof(double), cudaMemcpyHostToDevice, c->stream), "H2D");
+  CK(cudaMemcpyAsync(dlg, lg.data(), lg.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream), "H2D");
   CK(cudaMemcpyAsync(dbytes, q->nbytes, n * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream), "H2D");
   CK(cudaMemcpyAsync(dN, q->n_ranks, n * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream), "H2D");
   CK(cudaMemcpyAsync(dM, q->n_nodes, n * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream), "H2D");
@@ -2569,7 +2635,7 @@ int echo_cc_query(echo_ctx *c, const echo_cc_query_desc *q, double *out_ns) {
   CK(cudaMemcpyAsync(dalgo, q->cc_algo, n, cudaMemcpyHostToDevice, c->stream), "H2D");
   echo::ScenParams p{dprm, dprm + n, dprm + 2 * n, dprm + 3 * n, dprm + 4 * n, dprm + 5 * n};
   CK(timed(c, "cc_query", [&] {
-       return echo::launch_cc_query(n, dtype, dalgo, dbytes, dN, dM, dlg, p, tbl, dout, c->stream);
+       return echo::launch_cc_query(n, dtype, dalgo, dbytes, dN, dM, dlg, by_m, p, tbl, dout, c->stream);
      }), "cc_query launch");
   CK(cudaMemcpyAsync(out_ns, dout, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "D2H");
   CK(cudaStreamSynchronize(c->stream), "cc_query");

@@ -283,8 +283,10 @@ cudaError_t launch_cc_estimate(const CcSig *sig, int32_t G, ScenParams p, int32_
                                cudaStream_t st);
 cudaError_t launch_cc_scatter(const int32_t *comm_node, const int32_t *comm_sig, int64_t n_comm,
                               const int64_t *cc_dur, int32_t S, MatLayout lay, int64_t *dur, cudaStream_t st);
+cudaError_t launch_load_params(const double *const src[6], const double *slowdown, int32_t S, int32_t C, double *prm,
+                               double *sf, cudaStream_t st);
 cudaError_t launch_cc_query(int64_t n, const uint8_t *type, const uint8_t *algo, const int64_t *nbytes,
-                            const int32_t *N, const int32_t *M, const double *lg, ScenParams p,
+                            const int32_t *N, const int32_t *M, const double *lg, bool lg_by_m, ScenParams p,
                             const ChunkTable &tbl, double *out, cudaStream_t st);
 // sets *flag when row pairs[2p] of the [V][S] matrix `raw` (int32 or int64) differs
 // from row pairs[2p+1] in some scenario

@@ -156,6 +156,20 @@ __global__ void cc_scatter_kernel(const int32_t *__restrict__ comm_node, const i
   }
 }
 
+// The link parameters and slowdown factors of a batch, read where the caller has them:
+// blockIdx.y is the array.  Seven copies of a few KB took 2 to 9 us each.
+struct HostParams {
+  const double *link[6], *slowdown;
+};
+__global__ void load_params_kernel(HostParams h, int32_t S, int64_t n_sf, double *__restrict__ prm,
+                                   double *__restrict__ sf) {
+  const int k = blockIdx.y;
+  const double *src = k < 6 ? h.link[k] : h.slowdown;
+  double *dst = k < 6 ? prm + (int64_t)k * S : sf;
+  const int64_t n = k < 6 ? S : n_sf;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) dst[i] = src[i];
+}
+
 // A block's queries.  Every thread takes one as far as it is linear (send/recv and rings),
 // then the trees (a sixth of a mixed sweep) are gathered, so that two warps and not eight
 // run their code.  What bounds it is the fp64 pipe (divisions run at 73 G/s on this part):
@@ -478,10 +492,18 @@ cudaError_t launch_cc_scatter(const int32_t *comm_node, const int32_t *comm_sig,
 }
 
 cudaError_t launch_cc_query(int64_t n, const uint8_t *type, const uint8_t *algo, const int64_t *nbytes,
-                            const int32_t *N, const int32_t *M, const double *lg, ScenParams p,
+                            const int32_t *N, const int32_t *M, const double *lg, bool lg_by_m, ScenParams p,
                             const ChunkTable &tbl, double *out, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  cc_query_kernel<<<grid_for(n, kQueryThreads), kQueryThreads, 0, st>>>(n, Queries{type, algo, nbytes, N, M, lg, false, p}, tbl, out);
+  cc_query_kernel<<<grid_for(n, kQueryThreads), kQueryThreads, 0, st>>>(n, Queries{type, algo, nbytes, N, M, lg, lg_by_m, p}, tbl, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_load_params(const double *const src[6], const double *slowdown, int32_t S, int32_t C, double *prm,
+                               double *sf, cudaStream_t st) {
+  const HostParams h{{src[0], src[1], src[2], src[3], src[4], src[5]}, slowdown};
+  const dim3 grid((unsigned)std::min<int64_t>(((int64_t)std::max(1, C) * S + 255) / 256, 152), 7);
+  load_params_kernel<<<grid, 256, 0, st>>>(h, S, (int64_t)C * S, prm, sf);
   return cudaGetLastError();
 }
 

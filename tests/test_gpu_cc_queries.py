@@ -25,6 +25,8 @@ def _queries(rng, n, forms):
     q.n_ranks = np.where(rng.random(n) < 0.1, 1, q.n_ranks).astype(np.int32)
     q.n_nodes = np.where(q.n_ranks == 1, 1, q.n_nodes).astype(np.int32)
     q.n_nodes = np.minimum(q.n_nodes, q.n_ranks)
+    if n > 4000:  # more nodes than the table of logarithms holds
+        q.n_ranks[7], q.n_nodes[7] = 300_000, 5000
     return q
 
 
