@@ -2461,11 +2461,12 @@ int echo_read_times(echo_ctx *c, int64_t op0, int64_t op1, int32_t s0, int32_t s
   if ((rc = composition_status(c))) return rc;
   const int32_t Sr = s1 - s0;
   if (Sr == 0) return ECHO_OK;
+  const int64_t one_to_one = c->gb.V == c->gb.V_ext ? c->gb.V : -1;  // (a folded graph's ops stand for several)
   // Buffers of this device are written to directly: through the staging buffer every value
   // was written and read once more (GPT-175B x 250: 1.3 of 3.2 ms).
   if (device_buffer(c, start) && device_buffer(c, finish)) {
     CK(timed(c, "readback", [&] {
-         return echo::launch_readback(c->ext2int, op0, op1, s0, s1, c->lay, c->f[c->final_f], c->dur, c->cidx, c->lay_c,
+         return echo::launch_readback(c->ext2int, c->int2ext, one_to_one, op0, op1, s0, s1, c->lay, c->f[c->final_f], c->dur, c->cidx, c->lay_c,
                                       c->final_cd, start, finish, c->stream);
        }), "readback launch");
     CK(cudaStreamSynchronize(c->stream), "readback");
@@ -2480,7 +2481,7 @@ int echo_read_times(echo_ctx *c, int64_t op0, int64_t op1, int32_t s0, int32_t s
     int64_t *ds = static_cast<int64_t *>(c->stage);
     int64_t *df = ds + n;
     CK(timed(c, "readback", [&] {
-         return echo::launch_readback(c->ext2int, a, b, s0, s1, c->lay, c->f[c->final_f], c->dur, c->cidx, c->lay_c,
+         return echo::launch_readback(c->ext2int, c->int2ext, one_to_one, a, b, s0, s1, c->lay, c->f[c->final_f], c->dur, c->cidx, c->lay_c,
                                       c->final_cd, start ? ds : nullptr, finish ? df : nullptr, c->stream);
        }), "readback launch");
     if (start)

@@ -299,7 +299,8 @@ cudaError_t launch_compose(const ComposeArgs &a, int sigma, cudaStream_t st);
 cudaError_t launch_compose_staged(const StagedArgs &a, int sigma, const StagedPlan &plan, cudaStream_t st);
 cudaError_t launch_compose_levels(const LevelArgs &a, int sigma, cudaStream_t st);
 cudaError_t launch_overlap(const OverlapArgs &a, cudaStream_t st);
-cudaError_t launch_readback(const int32_t *ext2int, int64_t op0, int64_t op1, int32_t s0, int32_t s1, MatLayout lay,
+// V: the number of ops when int2ext takes them one to one to the caller's, else -1
+cudaError_t launch_readback(const int32_t *ext2int, const int32_t *int2ext, int64_t V, int64_t op0, int64_t op1, int32_t s0, int32_t s1, MatLayout lay,
                             const int64_t *f, const int64_t *d, const int32_t *cidx, MatLayout lay_c,
                             const int64_t *cd, int64_t *start, int64_t *finish, cudaStream_t st);
 cudaError_t launch_scatter_candidates(const int32_t *cand_node, int64_t n_cand, int32_t S, MatLayout lay,

@@ -423,6 +423,108 @@ __global__ void __launch_bounds__(256, 4) readback_tile_kernel(
   }
 }
 
+// The same when every op is asked for, of blocks of two scenarios and more, in columns of
+// kRingMinCols scenarios and more.  What bounds it is memory, and how whole the pieces are
+// that it is read and written in: tiles follow the internal order, so that a block's rows
+// come in pieces of 256 bytes and more, and leave as up to 2 KB of a caller's row each.  A
+// tile of both matrices comes into a ring in shared memory as it lies there (cp.async of 16
+// bytes, two tiles ahead); a block's part is padded by one row, so that a row of the tile is
+// read without bank conflicts.  Measured, all times of GPT-175B, tiles of 32 x 32 as above ->
+// this (us): x 200 1563 -> 1335, x 250 1880 -> 1502 (6.4 TB/s in the kernel), x 600 (three
+// columns of 200) 4180 -> 3999, x 1024 6795 -> 5802; columns of 176 (x 352) 2401 -> 2439,
+// of 150 (x 300) 2296 -> 2441.
+// Other tiles, x 250, kernel alone: 32 x 64 1787, 32 x 128 1514, 8 x 256 1695, 16 x 256 1380.
+// Blocks of one scenario (8-byte copies: x 100 891 -> 927) and ranges of ops (in the caller's
+// order a chain's few rows start and end inside a piece: x 250 1874 -> 1908) stay with the
+// kernel above.
+constexpr int kRingOps = 16, kRingCols = 256, kRingMinCols = 192, kRingStages = 3;
+constexpr int kRingTile = (kRingOps + 1) * kRingCols;  // elements of a padded tile of one matrix
+constexpr size_t kRingSmem = (size_t)kRingStages * 2 * kRingTile * sizeof(int64_t);
+// (blockIdx.y: `width` scenarios, a multiple of the block, from scenario c0 on)
+__global__ void __launch_bounds__(256) readback_all_kernel(const int32_t *__restrict__ int2ext, int64_t V, int32_t s0,
+                                                           int32_t s_end, int32_t width, MatLayout lay, const int64_t *__restrict__ f,
+                                                           const int64_t *__restrict__ d,
+                                                           const int32_t *__restrict__ cidx, MatLayout lay_c,
+                                                           const int64_t *__restrict__ cd, int64_t *__restrict__ start,
+                                                           int64_t *__restrict__ finish) {
+  constexpr int kCopies = kRingOps * kRingCols / 2 / 256, kEach = kRingOps * kRingCols / 256;
+  extern __shared__ __align__(16) int64_t tile[];  // [kRingStages][f, d][blocks][kRingOps + 1][block's scenarios]
+  __shared__ int32_t crow[4][kRingOps], to_row[4][kRingOps];  // candidate's row, caller's (-1: none)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int sl = lay.slog2, ul = sl - 1;  // (log2 of) a row's elements and copies
+  const int32_t c0 = (s0 >> sl << sl) + blockIdx.y * width, s1 = min(s_end, c0 + width);
+  const int64_t step = (int64_t)gridDim.x * kRingOps, first = (int64_t)blockIdx.x * kRingOps;
+  // this thread's copies of a tile: op (-1: none), place in the padded tile, scenario
+  int32_t op[kCopies], at[kCopies], scen[kCopies];
+#pragma unroll
+  for (int k = 0; k < kCopies; ++k) {
+    const int x = k * 256 + (int)threadIdx.x, blk = x / kRingOps >> ul, y = x & ((kRingOps << ul) - 1);
+    op[k] = y >> ul;
+    at[k] = (blk * (kRingOps + 1) << sl) + y * 2;
+    scen[k] = c0 + (blk << sl) + (y & ((1 << ul) - 1)) * 2;
+    if (scen[k] + 2 <= s0 || scen[k] >= s1) op[k] = -1;
+  }
+  // rows of tile t, by the first lanes of one warp
+  auto in = [&](int64_t t) { return lane < kRingOps && first + t * step + lane < V; };
+  auto cand = [&](int64_t t) { return cd && in(t) ? cidx[first + t * step + lane] : -1; };
+  auto outer = [&](int64_t t) { return in(t) ? int2ext[first + t * step + lane] : -1; };
+  auto put = [&](int64_t t, int32_t c, int32_t o) {
+    if (lane < kRingOps) crow[t & 3][lane] = c, to_row[t & 3][lane] = o;
+  };
+  auto load = [&](int64_t t) {
+    int64_t *const to = tile + (t % kRingStages) * 2 * kRingTile;
+#pragma unroll
+    for (int k = 0; k < kCopies; ++k) {
+      const int64_t i = first + t * step + op[k];
+      if (op[k] < 0 || i >= V) continue;
+      const int32_t ci = crow[t & 3][op[k]];
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(to + at[k]);
+      const int64_t from = lay.at(i, scen[k]);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(f + from) : "memory");
+      if (start)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + kRingTile * 8),
+                     "l"(ci >= 0 ? cd + lay_c.at(ci, scen[k]) : d + from)
+                     : "memory");
+    }
+  };
+  const int64_t tiles = first < V ? (V - first + step - 1) / step : 0;
+  int32_t c3 = -1, o3 = -1;  // rows of the tile three ahead
+  if (warp == 0) {
+    for (int t = 0; t < 3; ++t) put(t, cand(t), outer(t));
+    c3 = cand(3), o3 = outer(3);
+  }
+  __syncthreads();
+  for (int t = 0; t < kRingStages - 1; ++t) {
+    if (t < tiles) load(t);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  const int64_t Sr = s_end - s0;
+  const int32_t col = threadIdx.x, s = c0 + col;  // this thread's scenario
+  static_assert(kRingCols == 256, "a thread stores one column");
+  const bool mine = s >= s0 && s < s1;
+  const int from = ((col >> sl) * (kRingOps + 1) << sl) + (col & ((1 << sl) - 1));  // element (0, s) of a tile
+#pragma unroll 1
+  for (int64_t t = 0; t < tiles; ++t) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kRingStages - 2) : "memory");
+    __syncthreads();  // tile t is here for all, and tile t - 1 has been read by all
+    if (t + kRingStages - 1 < tiles) load(t + kRingStages - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (warp == 0) {
+      put(t + 3, c3, o3);
+      c3 = cand(t + 4), o3 = outer(t + 4);
+    }
+    const int64_t *const ft = tile + (t % kRingStages) * 2 * kRingTile + from, *const dt = ft + kRingTile;
+#pragma unroll
+    for (int o = 0; o < kEach; ++o) {
+      const int32_t r = to_row[t & 3][o];
+      if (r < 0 || !mine) continue;
+      const int64_t fv = ft[o << sl], to = r * Sr + (s - s0);
+      if (finish) finish[to] = fv;
+      if (start) start[to] = fv - dt[o << sl];
+    }
+  }
+}
+
 // Full validator durations for the kernels without a candidate ring: the
 // candidates' rows of the compact cd into dst (which holds the original durations).
 __global__ void scatter_candidates_kernel(const int32_t *__restrict__ cand_node, int64_t n_cand, int32_t S,
@@ -591,11 +693,23 @@ cudaError_t launch_overlap(const OverlapArgs &a, cudaStream_t st) {
   return prop ? launch_overlap_l0_p1(a, grid, tx, st) : launch_overlap_l0_p0(a, grid, tx, st);
 }
 
-cudaError_t launch_readback(const int32_t *ext2int, int64_t op0, int64_t op1, int32_t s0, int32_t s1, MatLayout lay,
+cudaError_t launch_readback(const int32_t *ext2int, const int32_t *int2ext, int64_t V, int64_t op0, int64_t op1, int32_t s0, int32_t s1, MatLayout lay,
                             const int64_t *f, const int64_t *d, const int32_t *cidx, MatLayout lay_c,
                             const int64_t *cd, int64_t *start, int64_t *finish, cudaStream_t st) {
   int64_t n = (op1 - op0) * (s1 - s0);
   if (n <= 0) return cudaSuccess;
+  // columns of one width, so that the blocks have the same to do; one wave of blocks, one on an SM
+  const int32_t sig = 1 << lay.slog2, S = s1 - (s0 & ~(sig - 1));
+  const int64_t cols = (S + kRingCols - 1) / kRingCols;
+  const int32_t width = (int32_t)((S + cols - 1) / cols + sig - 1) & ~(sig - 1);
+  if (op0 == 0 && op1 == V && width >= kRingMinCols && lay.slog2 >= 1 && lay.slog2 < 5) {
+    const int64_t tiles = (V + kRingOps - 1) / kRingOps;
+    const dim3 grid((unsigned)std::min<int64_t>(tiles, std::max<int64_t>(1, 152 / cols)), (unsigned)cols);
+    const cudaError_t e = cudaFuncSetAttribute(readback_all_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmem);
+    if (e != cudaSuccess) return e;
+    readback_all_kernel<<<grid, 256, kRingSmem, st>>>(int2ext, V, s0, s1, width, lay, f, d, cidx, lay_c, cd, start, finish);
+    return cudaGetLastError();
+  }
   if (s1 - s0 >= kReadCols && lay.slog2 < 5) {
     const int32_t first = s0 & ~(kReadCols - 1);
     const int64_t cols = (s1 - first + kReadCols - 1) / kReadCols, tiles = (op1 - op0 + kTileOps - 1) / kTileOps;

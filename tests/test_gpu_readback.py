@@ -1,4 +1,4 @@
-"""Reading times back from scenario blocks of every width: the tiled path (32 scenarios and more, blocks of 16 and fewer)
+"""Reading times back from scenario blocks of every width: the tiled paths (32 scenarios and more, columns of 192 and more)
 and the other one, op and scenario ranges that start and end inside tiles, host and device buffers; and the load's tiles
 and sums (32 and 64 bits), through the times they give."""
 import numpy as np
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("sigma", ["1", "2", "16", None])
-@pytest.mark.parametrize("S", [1, 33, 97])
+@pytest.mark.parametrize("S", [1, 33, 97, 401])
 def test_ranges_host_and_device(sigma, S, monkeypatch):
     import torch
 
