@@ -2224,9 +2224,11 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
     o.n_ranks = B.R;
     o.rows = B.V;
     o.c_rows = B.n_cand;
-    {  // pieces of each rank's list: enough warps for about eight waves (24 warps an SM; the
-       // pieces are not all of one length), each at least four batches of candidates long
-      const int64_t base = (int64_t)B.R * ((c->S + c->sigma - 1) / c->sigma), want = 8 * 24 * (int64_t)c->sms;
+    {  // pieces of each rank's list: enough warps for about four waves (24 warps an SM; the
+       // pieces are not all of one length, and each first looks for its place; with eight
+       // waves GPT-175B x 250 takes 334 us and not 300, with two x 1024 884 and not 774),
+       // each at least four batches of candidates long
+      const int64_t base = (int64_t)B.R * ((c->S + c->sigma - 1) / c->sigma), want = 4 * 24 * (int64_t)c->sms;
       const int64_t batch = (int64_t)echo::kOvBatch * (32 / c->sigma);
       o.parts = (int32_t)std::max<int64_t>(1, std::min((want + base - 1) / base, B.most_cands / (4 * batch)));
     }

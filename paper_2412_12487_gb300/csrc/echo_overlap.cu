@@ -81,10 +81,10 @@ __device__ __noinline__ int64_t launch_time(const int32_t *__restrict__ lq_off, 
 // What bounds it: with blocks of 8 scenarios and more, instructions (issue slots 60% busy
 // before the address arithmetic went to one multiply-add a load); with blocks of 1 and 2
 // memory, as a candidate's 8 or 16 bytes of a row cost 64.  Measured, before -> now (us):
-// GPT-1.3B x 1 80 -> 20, x 256 99 (blocks of 32; 123 in blocks of 2) -> 75, x 500 folded
+// GPT-1.3B x 1 80 -> 20, x 256 99 (blocks of 32; 123 in blocks of 2) -> 69, x 500 folded
 // 330 -> 35 (its pieces are now cut by the longest rank's list, not the mean of all ranks);
-// GPT-175B x 250 338 (blocks of 32; 535 in blocks of 2) -> 347, x 1024 1050 -> 790; 1024
-// ranks x 64 1000 -> 765.
+// GPT-175B x 250 338 (blocks of 32; 535 in blocks of 2) -> 306, x 1024 1050 -> 780; 1024
+// ranks x 64 1000 -> 678.
 // LAUNCH: a comm op's interval on the rank opens at the rank's launch of it
 // (a.lq_off), else at its start.  PROP: the proportional slowdown model.
 template <int NCMAX, bool LAUNCH, bool PROP>
@@ -144,14 +144,6 @@ __global__ void __launch_bounds__(kOvWarps * 32, overlap_min_blocks(NCMAX, LAUNC
       sw[j] = launch_time(a.lq_off, a.lq_ops, f, sh, cur[j]);
     } else {
       sw[j] = fw[j] - du[w << sh];
-    }
-  };
-  auto seek = [&](int j) {  // cursor j at position cur[j]
-    if (cur[j] < end[j]) {
-      fetch(j, a.cq_ops[cur[j]]);
-      nid[j] = cur[j] + 1 < end[j] ? a.cq_ops[cur[j] + 1] : 0;
-    } else {
-      sw[j] = fw[j] = INT64_MAX;
     }
   };
   auto advance = [&](int j) {  // cursor j one position on
@@ -214,37 +206,84 @@ __global__ void __launch_bounds__(kOvWarps * 32, overlap_min_blocks(NCMAX, LAUNC
         sv0 = f[(int64_t)q.x << sh] - (cu ? cu[(int64_t)q.y << sh] : du[(int64_t)q.x << sh]);
       }
     }
+    // binary searches (first comm op finishing after sv0; finishes are sorted): of many
+    // timelines side by side, so that a round waits for memory twice and not twice a timeline
+    // (1024 ranks x 64: 767 -> 709 us); of few one after the other, which
+    // needs fewer registers (GPT-1.3B x 45, launch intervals: 47 us, side by side 51)
+    constexpr bool kTogether = NCMAX > 4;
+    const bool inner = part > 0 || team > 0;
+    int32_t hi[NCMAX];
 #pragma unroll
     for (int j = 0; j < NCMAX; ++j) {
-      cur[j] = end[j] = 0;
+      cur[j] = j < nc ? (int32_t)a.cq_off[r * nc + j] : 0;
+      end[j] = j < nc ? (int32_t)a.cq_off[r * nc + j + 1] : 0;
+      hi[j] = inner ? end[j] : cur[j];
       sw[j] = fw[j] = INT64_MAX;
-      if (j < nc) {
-        int32_t lo = (int32_t)a.cq_off[r * nc + j], hi = (int32_t)a.cq_off[r * nc + j + 1];
-        end[j] = hi;
-        if (part > 0 || team > 0) {
-          while (lo < hi) {  // first comm op finishing after sv0 (finishes are sorted)
-            const int32_t mid = (lo + hi) >> 1;
-            if (a.dbg && !in_range(a.cq_ops[mid], a.rows)) {  // debug bounds: stop searching
-              atomicCAS(a.status, 0, (int32_t)kDevBounds);
-              break;
-            }
-            if (f[(int64_t)a.cq_ops[mid] << sh] > sv0)
-              hi = mid;
-            else
-              lo = mid + 1;
+    }
+    auto search = [&](int j) { return cur[j] < hi[j]; };
+#pragma unroll
+    for (int j = 0; j < NCMAX; ++j)
+      while (!kTogether && search(j)) {
+        const int32_t mid = (cur[j] + hi[j]) >> 1, w = a.cq_ops[mid];
+        if (a.dbg && !in_range(w, a.rows)) {  // debug bounds: stop searching
+          atomicCAS(a.status, 0, (int32_t)kDevBounds);
+          hi[j] = cur[j];
+        } else if (f[(int64_t)w << sh] > sv0) {
+          hi[j] = mid;
+        } else {
+          cur[j] = mid + 1;
+        }
+      }
+    while (kTogether) {
+      bool any = false;
+#pragma unroll
+      for (int j = 0; j < NCMAX; ++j)
+        if (search(j)) {
+          any = true;
+          nid[j] = a.cq_ops[(cur[j] + hi[j]) >> 1];
+          if (a.dbg && !in_range(nid[j], a.rows)) {  // debug bounds: stop searching
+            atomicCAS(a.status, 0, (int32_t)kDevBounds);
+            hi[j] = cur[j];
           }
         }
-        cur[j] = lo;
-        seek(j);
-        while (cur[j] < end[j] && sw[j] >= fw[j]) advance(j);  // zero-length ops never overlap
-      }
+      if (!any) break;
+#pragma unroll
+      for (int j = 0; j < NCMAX; ++j)
+        if (search(j)) fw[j] = f[(int64_t)nid[j] << sh];
+#pragma unroll
+      for (int j = 0; j < NCMAX; ++j)
+        if (search(j)) {
+          const int32_t mid = (cur[j] + hi[j]) >> 1;
+          if (fw[j] > sv0)
+            hi[j] = mid;
+          else
+            cur[j] = mid + 1;
+        }
     }
+#pragma unroll
+    for (int j = 0; j < NCMAX; ++j)
+      if (cur[j] < end[j]) nid[j] = a.cq_ops[cur[j]];
+#pragma unroll
+    for (int j = 0; j < NCMAX; ++j) {
+      if (cur[j] < end[j])
+        fetch(j, nid[j]);
+      else
+        sw[j] = fw[j] = INT64_MAX;
+    }
+#pragma unroll
+    for (int j = 0; j < NCMAX; ++j) nid[j] = cur[j] + 1 < end[j] ? a.cq_ops[cur[j] + 1] : 0;
+#pragma unroll
+    for (int j = 0; j < NCMAX; ++j)
+      while (cur[j] < end[j] && sw[j] >= fw[j]) advance(j);  // zero-length ops never overlap
   }
   // The smallest cursor end and start over the timelines: while every cursor op
   // ends after a candidate starts (fmin > sv), no cursor moves, and the candidate
   // overlaps iff some cursor op starts before it ends (smin < fv).
+  // (Up to four timelines are compared one by one: as many instructions, and none a move.)
+  constexpr bool kDirect = NCMAX <= 4;
   int64_t fmin, smin;
   auto bounds = [&]() {
+    if (kDirect) return;
     fmin = smin = INT64_MAX;
 #pragma unroll
     for (int j = 0; j < NCMAX; ++j)
@@ -269,10 +308,15 @@ __global__ void __launch_bounds__(kOvWarps * 32, overlap_min_blocks(NCMAX, LAUNC
     for (int32_t i = i0 + team, u = 0; u < kOvBatch && i < last; ++u, i += teams, rec += rec_step, val += kValStep) {
       const int64_t fv = s_ld64(val), dv = s_ld64(val + 256), sv = fv - dv;
       const uint4 q = s_ld128(rec);
-      if (fmin <= sv) {
+      bool move = !kDirect && fmin <= sv;
+      if (kDirect) {
+#pragma unroll
+        for (int j = 0; j < NCMAX; ++j) move |= fw[j] <= sv;
+      }
+      if (move) {
 #pragma unroll
         for (int j = 0; j < NCMAX; ++j) {
-          if (j < nc && fw[j] <= sv) {  // the cursor op ended before this op starts: move on
+          if (fw[j] <= sv) {  // the cursor op ended before this op starts: move on
             do {
               advance(j);
             } while (cur[j] < end[j] && (fw[j] <= sv || sw[j] >= fw[j]));
@@ -280,7 +324,12 @@ __global__ void __launch_bounds__(kOvWarps * 32, overlap_min_blocks(NCMAX, LAUNC
         }
         bounds();
       }
-      const bool hit = smin < fv && sv < fv;
+      bool hit = !kDirect && smin < fv;
+      if (kDirect) {
+#pragma unroll
+        for (int j = 0; j < NCMAX; ++j) hit |= sw[j] < fv;
+      }
+      hit &= sv < fv;
       int64_t len = 0;
       if (PROP && hit && cn) {
         // proportional model: the length of [sv, fv) covered by the union of the
