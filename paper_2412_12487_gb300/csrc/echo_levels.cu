@@ -26,8 +26,8 @@
 // Measured, first / final composition (us), before -> now:
 //   GPT-1.3B x 1      415 / 453   ->  138 / 143   (dataflow composer before)
 //   GPT-1.3B x 256    415 / 461   ->  159 / 180   (dataflow composer before)
-//   GPT-175B x 250   2895 / 3099  -> 1060 / 1210  (dataflow composer before)
-//   GPT-175B x 1024  3362 / 3731  -> 2200 / 3240
+//   GPT-175B x 250   2895 / 3099  -> 1060 / 1200  (dataflow composer before)
+//   GPT-175B x 1024  3362 / 3731  -> 2110 / 3100
 #include <cuda_runtime.h>
 
 #include <cstdint>
