@@ -78,9 +78,10 @@ __device__ __noinline__ int64_t launch_time(const int32_t *__restrict__ lq_off, 
 // overlapped compute op of positive length gets rint(d * slowdown) or the proportional
 // form for the next composition (cd_next, compact); the decisions themselves are stored
 // only when `ov` is given.
-// What bounds it: with blocks of 8 scenarios and more, instructions (issue slots 60% busy
-// before the address arithmetic went to one multiply-add a load); with blocks of 1 and 2
-// memory, as a candidate's 8 or 16 bytes of a row cost 64.  Measured, before -> now (us):
+// What bounds it: instructions (issue slots half busy and more); with blocks of 1 and 2 each
+// team's own search and cursor moves, which the warp runs one after the other.  (Starts and
+// finishes in compact matrices of their own: 316 against 306 us on GPT-175B x 250, and the
+// composition that writes them 1212 against 1062.)  Measured, before -> now (us):
 // GPT-1.3B x 1 80 -> 20, x 256 99 (blocks of 32; 123 in blocks of 2) -> 69, x 500 folded
 // 330 -> 35 (its pieces are now cut by the longest rank's list, not the mean of all ranks);
 // GPT-175B x 250 338 (blocks of 32; 535 in blocks of 2) -> 306, x 1024 1050 -> 780; 1024
