@@ -1826,8 +1826,10 @@ int echo_create(echo_ctx **out, int device, void *cuda_stream) {
     }
     c->own_stream = true;
   }
-  int pageable = 0;
-  c->reads_host = cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, device) == cudaSuccess && pageable;
+  // (through the host's page tables; where pages would migrate instead, copies are better)
+  int in_place = 0;
+  c->reads_host = cudaDeviceGetAttribute(&in_place, cudaDevAttrPageableMemoryAccessUsesHostPageTables, device) ==
+                      cudaSuccess && in_place && !std::getenv("ECHO_TEST_COPY_INPUTS");  // (tests: the other path)
   if (const char *e = std::getenv("ECHO_COMPOSE_KERNEL")) {  // tuning and tests: force a compose kernel
     const std::string k(e);
     c->kernel_choice = k == "direct" ? 1 : k == "staged" ? 2 : k == "pipelined" ? 3 : k == "dataflow" ? 4 : 0;

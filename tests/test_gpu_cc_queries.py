@@ -49,8 +49,12 @@ FORMS = {"mixed": [(0, 0), (0, 1), (0, 2), (1, 0), (2, 0), (3, 0)], "trees": [(0
 @pytest.mark.parametrize("forms", list(FORMS))
 @pytest.mark.parametrize("n", [1, 31, 255, 256, 257, 5000])
 @pytest.mark.parametrize("table", TABLES, ids=["default", "bytes", "wide"])
-def test_queries_equal_the_oracle(forms, n, table):
+@pytest.mark.parametrize("copies", [False, True])
+def test_queries_equal_the_oracle(forms, n, table, copies, monkeypatch):
     import torch
+
+    if copies:  # host arrays uploaded, not read in place
+        monkeypatch.setenv("ECHO_TEST_COPY_INPUTS", "1")
 
     q = _queries(np.random.default_rng(n), n, FORMS[forms])
     want = _want(q, table)
@@ -72,3 +76,23 @@ def test_queries_equal_the_oracle(forms, n, table):
         assert lib.echo_cc_query_noalloc(C.byref(d), C.c_void_p(t.data_ptr()),
                                          C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
         assert np.array_equal(t.cpu().numpy(), want)
+
+
+def test_parameters_uploaded_or_read_in_place(monkeypatch):
+    c = W.GPTConfig(**{**W.config("tiny").__dict__, "fixed_scenario": False})
+    g = W.build_gpt_graph(c)
+    for S in (1, 7, 300):
+        sc = W.make_scenarios(g, c, n_scen=S)
+        want = oracle.compose(g, sc)
+        for copies in (False, True):
+            if copies:
+                monkeypatch.setenv("ECHO_TEST_COPY_INPUTS", "1")
+            else:
+                monkeypatch.delenv("ECHO_TEST_COPY_INPUTS", raising=False)
+            with E.Echo(0) as e:
+                e.load_graph(g)
+                e.load_scenarios(sc)
+                e.estimate_collectives()
+                e.compose()
+                assert np.array_equal(e.read_makespan(), want.makespan)
+                assert np.array_equal(e.read_times()[1], want.finish)
