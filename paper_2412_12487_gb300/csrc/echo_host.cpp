@@ -1615,6 +1615,10 @@ void free_all(std::vector<void *> &v) {
   v.clear();
 }
 
+// A context starts with this much: small calls never wait for an allocation (the first of a
+// process maps 2 MB, 60 us).
+constexpr size_t kStageStart = 1 << 20;
+
 int stage_reserve(echo_ctx *c, size_t bytes) {
   if (c->stage_bytes >= bytes) return ECHO_OK;
   if (c->stage) cudaFree(c->stage);
@@ -1825,6 +1829,11 @@ int echo_create(echo_ctx **out, int device, void *cuda_stream) {
       return ECHO_E_CUDA;
     }
     c->own_stream = true;
+  }
+  if (stage_reserve(c, kStageStart) != ECHO_OK) {
+    if (c->own_stream) cudaStreamDestroy(c->stream);
+    delete c;
+    return ECHO_E_OOM;
   }
   // (through the host's page tables; where pages would migrate instead, copies are better)
   int in_place = 0;
@@ -2579,7 +2588,8 @@ int echo_cc_query(echo_ctx *c, const echo_cc_query_desc *q, double *out_ns) {
   if ((rc = check_params(c, n, q->alpha_ns, q->bw_intra, q->lat_intra, q->bw_inter, q->lat_inter, q->delta))) return rc;
   ChunkTable tbl;
   if ((rc = make_table(c, q->n_chunk, q->chunk_max_bytes, q->chunk_bytes, &tbl))) return rc;
-  // log2(M): a table by M, or one a query where groups span more nodes than that
+  // log2(M): a table by M, or one a query where groups span more nodes than the table or
+  // than there are queries
   constexpr int32_t kMaxTable = 4096;
   int64_t bad = 0;
   int32_t max_m = 0;
@@ -2597,9 +2607,15 @@ int echo_cc_query(echo_ctx *c, const echo_cc_query_desc *q, double *out_ns) {
     if (q->nbytes[i] < 0 || q->n_ranks[i] < 1 || q->n_nodes[i] < 1 || q->n_nodes[i] > q->n_ranks[i])
       return set_err(c, ECHO_E_INVALID_ARG, "query " + std::to_string(i) + ": need bytes >= 0 and 1 <= M <= N");
   }
-  const bool by_m = max_m <= kMaxTable;
-  std::vector<double> lg(by_m ? (size_t)max_m + 1 : (size_t)n, 0.0);
-  for (size_t i = by_m ? 1 : 0; i < lg.size(); ++i) lg[i] = std::log2((double)(by_m ? (int32_t)i : q->n_nodes[i]));
+  const bool by_m = max_m <= kMaxTable && max_m <= n;
+  std::vector<double> lg(by_m ? (size_t)max_m + 1 : (size_t)n, 0.0), seen;
+  for (int32_t m = 1; by_m && m <= max_m; ++m) lg[m] = std::log2((double)m);
+  if (!by_m) seen.assign(kMaxTable + 1, -1.0);
+  for (int64_t i = 0; !by_m && i < n; ++i) {
+    const int32_t m = q->n_nodes[i];
+    if (m <= kMaxTable && seen[m] < 0) seen[m] = std::log2((double)m);
+    lg[i] = m <= kMaxTable ? seen[m] : std::log2((double)m);
+  }
   const double *src[6] = {q->alpha_ns, q->bw_intra, q->lat_intra, q->bw_inter, q->lat_inter, q->delta};
   if (c->reads_host) {
     // The kernel reads the caller's arrays where they are: of the 290 us that 20011 queries
