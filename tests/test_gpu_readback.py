@@ -42,6 +42,9 @@ def test_ranges_host_and_device(sigma, S, monkeypatch):
                         assert rc == 0
                     assert np.array_equal(ds.cpu().numpy(), want.start[op0:op1, s0:s1])
                     assert np.array_equal(df.cpu().numpy(), want.finish[op0:op1, s0:s1])
+        dm = torch.full((S,), -1, dtype=torch.int64, device="cuda")
+        assert e.lib.echo_read_makespan(e.h, dm.data_ptr()) == 0
+        assert np.array_equal(dm.cpu().numpy(), want.makespan) and np.array_equal(e.read_makespan(), want.makespan)
         bad = sc.dur.copy()
         bad[np.nonzero(g.kind == W.KIND_COMPUTE)[0][-1], S - 1] = -1
         with pytest.raises(EchoError) as ei:
