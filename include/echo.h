@@ -17,7 +17,8 @@
  *     context keeps its previous state and echo_last_error() describes the cause.
  *   - Array arguments are caller-owned HOST memory unless stated otherwise.  They
  *     are read (or written) during the call only; nothing keeps a pointer to them.
- *     Pinned (page-locked) host memory makes the copies faster but is not required.
+ *     Pinned (page-locked) host memory makes the copies faster but is not required,
+ *     and neither is any alignment.
  *   - Op ids are the caller's ids 0..n_ops-1.  The library renumbers internally
  *     and never exposes its own numbering.
  *   - Times are int64 nanoseconds; the first op of every timeline may start at 0.

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "echo.h"
+#include "echo_align.h"
 #include "echo_internal.h"
 
 using echo::CcSig;
@@ -1519,7 +1520,7 @@ struct echo_ctx {
   // `small`, so that each call reads its status and results back with one copy
   int64_t *small = nullptr;
   std::vector<int64_t> h_small;
-  bool reads_host = false;  // kernels may read the caller's host arrays in place (a coherent link to its memory)
+  bool reads_host = false;  // kernels may read the caller's host arrays in place (a coherent link to its memory), where aligned
   int32_t *status = nullptr;
   // scenarios
   int32_t S = 0, C = 0, sigma = 1;
@@ -2127,7 +2128,9 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
   c->h_maxsf = maxsf;
   // parameters
   const double *src[6] = {sc->alpha_ns, sc->bw_intra, sc->lat_intra, sc->bw_inter, sc->lat_inter, sc->delta};
-  if (!c->reads_host) {
+  const bool in_place =
+      c->reads_host && echo::elements_aligned(sizeof(double), {src[0], src[1], src[2], src[3], src[4], src[5], sc->slowdown});
+  if (!in_place) {
     for (int k = 0; k < 6; ++k)
       CK(cudaMemcpyAsync(c->prm + (size_t)k * S, src[k], S * sizeof(double), cudaMemcpyHostToDevice, c->stream), "parameter upload");
     CK(cudaMemcpyAsync(c->sf, sc->slowdown, (size_t)C * S * sizeof(double), cudaMemcpyHostToDevice, c->stream),
@@ -2142,7 +2145,7 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
   }
   // (one launch that reads the caller's arrays, and from here on no way out before the wait)
   const cudaError_t loaded =
-      c->reads_host ? echo::launch_load_params(src, sc->slowdown, S, C, c->prm, c->sf, c->stream) : cudaSuccess;
+      in_place ? echo::launch_load_params(src, sc->slowdown, S, C, c->prm, c->sf, c->stream) : cudaSuccess;
   int32_t st = 0;
   if ((rc = read_small(c, 0, 2 * (int64_t)S + 1, &st))) return rc;
   CK(loaded, "parameter upload");
@@ -2617,7 +2620,8 @@ int echo_cc_query(echo_ctx *c, const echo_cc_query_desc *q, double *out_ns) {
     lg[i] = m <= kMaxTable ? seen[m] : std::log2((double)m);
   }
   const double *src[6] = {q->alpha_ns, q->bw_intra, q->lat_intra, q->bw_inter, q->lat_inter, q->delta};
-  if (c->reads_host) {
+  if (c->reads_host && echo::elements_aligned(sizeof(double), {src[0], src[1], src[2], src[3], src[4], src[5]}) &&
+      echo::elements_aligned(sizeof(int64_t), {q->nbytes}) && echo::elements_aligned(sizeof(int32_t), {q->n_ranks, q->n_nodes})) {
     // The kernel reads the caller's arrays where they are: of the 290 us that 20011 queries
     // took, the twelve uploads were 105 (9 each, one after the other), the checks 100
     // (with a branch a field), the kernel 11.
