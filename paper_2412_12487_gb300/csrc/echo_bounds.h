@@ -23,6 +23,12 @@ ECHO_HD bool in_range(int64_t i, int64_t n) { return i >= 0 && i < n; }
 // [lo, hi) is a (possibly empty) sub-range of [0, n)
 ECHO_HD bool range_ok(int64_t lo, int64_t hi, int64_t n) { return 0 <= lo && lo <= hi && hi <= n; }
 
+// the n elements from `first` on are elements of [0, total), and `first` is a multiple of
+// `align` (vector loads of shared memory)
+ECHO_HD bool place_ok(int64_t first, int64_t n, int64_t align, int64_t total) {
+  return range_ok(first, first + n, total) && first % align == 0;
+}
+
 // the k-th set bit below position t of a 64-bit chain mask, counted from a first
 // index `first`, is an element of [0, n): the compact row of a masked chain position
 ECHO_HD bool masked_row_ok(int64_t first, uint64_t mask, int64_t n) {

@@ -162,6 +162,19 @@ __device__ __forceinline__ void lv_bad(const Shared &sh, const LevelArgs &a) {  
   atomicCAS(a.status, (int32_t)kDevOk, (int32_t)kDevBounds);
 }
 
+// Debug bounds: what a step's descriptor places (records and masks, duration rows, starts,
+// candidates' rows and the row list) lies in the ring, at the alignment that it is read
+// with, and its rows in the matrix.  (Out of line: the checking variant only.)
+template <int SIGMA>
+__device__ __noinline__ bool desc_ok(const LevelArgs &a, const uint4 &m, const uint4 &m2) {
+  constexpr uint32_t kRow = SIGMA * 8, kVec = SIGMA >= 2 ? 16 : 8;
+  const int64_t segs = m.y & 0xFFFF, rows = m.y >> 16, cands = m2.x >> 16, R = a.ring_bytes;
+  const int64_t recs = cands ? ((4 * segs + 15) & ~15) + 16 * segs : 4 * segs;
+  return place_ok(m.x, recs, 16, R) && place_ok(m.z, rows * kRow, kVec, R) && place_ok(m.w, segs * kRow, kVec, R) &&
+         (!cands || place_ok(m2.z, cands * kRow, kVec, R)) && (level_walks(SIGMA) || place_ok(m2.w, 2 * rows, 2, R)) &&
+         range_ok(m2.y, m2.y + rows, a.pitch);
+}
+
 // ---- copy warps: kLvCopyWarps of them take the levels in turn ------------------------
 // A bulk copy costs its issuing thread about 220 cycles and each further one right after
 // it 50, and the fence 250 while other warps store to global memory (measured apart from
@@ -204,7 +217,8 @@ __device__ void copy_role(const LevelArgs &a, const Shared &sh, int c, int lane)
       if (DBG && !(range_ok(r.z, (int64_t)r.z + r.w, n_recs) && range_ok(d.z, (int64_t)d.z + d.w, a.pitch) &&
                    (!a.cdur || range_ok(q.z, (int64_t)q.z + q.w, a.c_pitch)) &&
                    range_ok(r.x, (int64_t)r.x + b_rec, a.ring_bytes) && range_ok(d.x, (int64_t)d.x + b_dur, a.ring_bytes) &&
-                   range_ok(q.x, (int64_t)q.x + b_cand, a.ring_bytes) && dep < l)) {
+                   range_ok(q.x, (int64_t)q.x + b_cand, a.ring_bytes) && (r.x | d.x | (b_cand ? q.x : 0)) % 16 == 0 &&
+                   (d.z | d.w | (a.cdur ? q.z | q.w : 0)) * SIGMA % 2 == 0 && dep < l)) {
         lv_bad(sh, a);
         ok = false;
         break;
@@ -367,7 +381,12 @@ __device__ void sum_role(const LevelArgs &a, const Shared &sh, int team, int tea
     if (!__all_sync(0xffffffffu, lv_wait(sh.full + (l & kStageMask), l / kLvStages, sh, a))) return;
     const uint32_t ds = desc_of(sh, l);
     const uint4 m = s_ld128(ds);
-    const uint32_t nseg = m.y & 0xFFFF, recs = sh.ring + m.x, dur = sh.ring + m.z + j;
+    uint32_t nseg = m.y & 0xFFFF;
+    const uint32_t recs = sh.ring + m.x, dur = sh.ring + m.z + j;
+    if (DBG && !desc_ok<SIGMA>(a, m, s_ld128(ds + 16))) {
+      lv_bad(sh, a);
+      nseg = 0;
+    }
 #pragma unroll 1
     for (uint32_t k = sw; k < nseg; k += (uint32_t)nw * SPW) {
       const uint32_t h = s_ld32(recs + 4 * k);
@@ -446,10 +465,15 @@ __device__ void head_role(const LevelArgs &a, const Shared &sh, int t, int nt, i
 #pragma unroll
   for (int i = 0; i < LV; ++i) mk[i] = 0;
   bool ok = true;
+  // debug bounds: a place of `n` values in shared memory, aligned as it is read
+  auto inside = [&](uint32_t place, int64_t n, uint32_t align) {
+    return place_ok(place, n, align, a.smem_bytes / 8);
+  };
+  constexpr uint32_t kZero = kLvFixedBytes / 8;  // slot 0
   auto row = [&](uint32_t place, int64_t (&x)[LV]) {
-    if (DBG && !in_range(place, a.smem_bytes / 8)) {
+    if (DBG && !inside(place, SIGMA, LV)) {
       lv_bad(sh, a);
-      place = 0;
+      place = kZero;
     }
     s_load<LV>(at + place * 8, x);
   };
@@ -473,12 +497,17 @@ __device__ void head_role(const LevelArgs &a, const Shared &sh, int t, int nt, i
     top(s, u);
     top(v, w);
     top(s, v);
-    if (h.w >> 16) {  // a list: pieces of 16 bytes, the first {pieces, six inputs}, the others eight inputs
-      uint32_t e = sh.base + (h.w >> 16) * 8;
+    uint32_t more = h.w >> 16;
+    if (DBG && more && !inside(more, 2, 2)) {  // (its first piece, before that is read)
+      lv_bad(sh, a);
+      more = 0;
+    }
+    if (more) {  // a list: pieces of 16 bytes, the first {pieces, six inputs}, the others eight inputs
+      uint32_t e = sh.base + more * 8;
       uint4 y = s_ld128(e);
       uint32_t n = y.x;
       y.x = 0;
-      if (DBG && !range_ok((h.w >> 16) * 8, (int64_t)(h.w >> 16) * 8 + 16 * (int64_t)n, a.smem_bytes)) {
+      if (DBG && !(n > 0 && inside(more, 2 * (int64_t)n, 2))) {
         lv_bad(sh, a);
         n = 1;
       }
@@ -502,7 +531,7 @@ __device__ void head_role(const LevelArgs &a, const Shared &sh, int t, int nt, i
     int64_t f[LV];
 #pragma unroll
     for (int i = 0; i < LV; ++i) f[i] = s[i] + sum[i];
-    if (DBG && !(in_range(h.x >> 16, a.smem_bytes / 8) && in_range(h.y & 0xFFFF, a.smem_bytes / 8))) {
+    if (DBG && !(inside(h.x >> 16, SIGMA, LV) && inside(h.y & 0xFFFF, SIGMA, LV))) {
       lv_bad(sh, a);
       return;
     }
@@ -550,7 +579,11 @@ __device__ void walk_role(const LevelArgs &a, const Shared &sh, int team, int te
     const uint32_t ds = desc_of(sh, l);
     const uint4 m = s_ld128(ds), m2 = s_ld128(ds + 16);
     const uint32_t nseg = m.y & 0xFFFF, recs = sh.ring + m.x, dur = sh.ring + m.z + j;
-    const uint32_t n = ALL ? nseg : m2.x & 0xFFFF;
+    uint32_t n = ALL ? nseg : m2.x & 0xFFFF;
+    if (DBG && !desc_ok<SIGMA>(a, m, m2)) {
+      lv_bad(sh, a);
+      n = 0;
+    }
 #pragma unroll 1
     for (uint32_t x = sw; x < n; x += (uint32_t)nw * SPW) {
       uint32_t k = x, len, h;
@@ -638,7 +671,11 @@ __device__ void store_role(const LevelArgs &a, const Shared &sh, int team, int t
     const uint32_t ds = desc_of(sh, l);
     const uint4 m = s_ld128(ds), m2 = s_ld128(ds + 16);
     const uint32_t counts = m.y, row0 = m2.y, map = sh.ring + m2.w, start = sh.ring + m.w, dur = sh.ring + m.z;
-    const uint32_t n = (ALL ? counts >> 16 : m2.x & 0xFFFF) * VPR;  // vectors
+    uint32_t n = (ALL ? counts >> 16 : m2.x & 0xFFFF) * VPR;  // vectors
+    if (DBG && !desc_ok<SIGMA>(a, m, m2)) {
+      lv_bad(sh, a);
+      n = 0;
+    }
     int64_t *fl = fb + (int64_t)row0 * SIGMA;
     // vector x: its row of the level and its segment; the loads of 4 vectors are in flight together
 #pragma unroll 1
@@ -659,7 +696,7 @@ __device__ void store_role(const LevelArgs &a, const Shared &sh, int team, int t
           }
           if (DBG && !(in_range(row[u], counts >> 16) && in_range(seg[u], counts & 0xFFFF))) {
             lv_bad(sh, a);
-            row[u] = seg[u] = 0;
+            n = 0;  // (row and segment 0 need not exist)
           }
         }
       }

@@ -54,6 +54,31 @@ int main() {
 """
 
 
+PLACES = r"""
+#include <stdio.h>
+#include "echo_bounds.h"
+using echo::place_ok;
+int main() {
+  int bad = 0;
+  // pieces of two values in 100 of them: a list of inputs at the very end, past it, and at an odd place
+  for (int at = -3; at < 110; ++at)
+    for (int n = 0; n < 5; ++n)
+      for (int align : {1, 2, 16}) bad += place_ok(at, n, align, 100) != (at >= 0 && at + n <= 100 && at % align == 0);
+  bad += place_ok(65535, 2, 1, 232448 / 8);  // the largest 16-bit place lies beyond a block's shared memory
+  bad += place_ok(98, 2 * (int64_t)UINT32_MAX, 2, 100);
+  return bad;
+}
+"""
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+def test_places_in_shared_memory(tmp_path):
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text(PLACES)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(exe)])
+    assert subprocess.run([str(exe)]).returncode == 0
+
+
 @pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
 def test_bounds_predicates_on_the_host():
     with tempfile.TemporaryDirectory() as d:

@@ -58,3 +58,25 @@ def test_chain_and_join_edges_bit_exact(sigma, ranks, monkeypatch):
                 assert got["info"]["sigma"] == sigma
                 want = oracle.compose(g, sc, refine_passes=refine, overlap_model=model, comm_interval=interval)
                 assert_same(got, want, g, refine)
+
+
+@pytest.mark.parametrize("sigma", [1, 2, 4, 8, 16])
+def test_debug_bounds_of_every_block_width(sigma, monkeypatch):
+    """The checking variant of every role (sums in place and stores by rows for blocks of 1 and 2, walks above; lists of
+    inputs; candidates): no check fails on well-formed graphs, and the times are the oracle's."""
+    monkeypatch.setenv("ECHO_COMPOSE_KERNEL", "pipelined")
+    monkeypatch.setenv("ECHO_SIGMA", str(sigma))
+    rng = np.random.default_rng(300 + sigma)
+    graphs = [_joins(11, [1, 3, 64, 65]), _joins(150, [1, 9, 12])]
+    graphs += [SG.random_graph(rng, int(rng.integers(20, 300)), max_ranks=5, max_streams=8, p_edge=0.03) for _ in range(4)]
+    with Echo(0) as e:
+        for g in graphs:
+            sc = SG.random_scenarios(rng, g, sigma + 1, max_dur=20_000)
+            for refine, model, interval in ((0, 0, 0), (2, 1, 1)):
+                e.load_graph(g)
+                e.load_scenarios(sc)
+                e.estimate_collectives()
+                e.compose(refine_passes=refine, overlap_model=model, comm_interval=interval, debug_bounds=True)
+                st, fn = e.read_times()
+                got = dict(start=st, finish=fn, makespan=e.read_makespan(), cc=e.read_cc(), ov=e.read_overlap())
+                assert_same(got, oracle.compose(g, sc, refine_passes=refine, overlap_model=model, comm_interval=interval), g, refine)
