@@ -55,6 +55,7 @@ int main() {
 
 
 PLACES = r"""
+#include <initializer_list>
 #include <stdio.h>
 #include "echo_bounds.h"
 using echo::place_ok;
