@@ -698,11 +698,12 @@ cudaError_t launch_readback(const int32_t *ext2int, const int32_t *int2ext, int6
                             const int64_t *cd, int64_t *start, int64_t *finish, cudaStream_t st) {
   int64_t n = (op1 - op0) * (s1 - s0);
   if (n <= 0) return cudaSuccess;
+  constexpr int64_t kMaxCols = 65535;  // columns of the tiled kernels (the grid's second dimension)
   // columns of one width, so that the blocks have the same to do; one wave of blocks, one on an SM
   const int32_t sig = 1 << lay.slog2, S = s1 - (s0 & ~(sig - 1));
   const int64_t cols = (S + kRingCols - 1) / kRingCols;
   const int32_t width = (int32_t)((S + cols - 1) / cols + sig - 1) & ~(sig - 1);
-  if (op0 == 0 && op1 == V && width >= kRingMinCols && lay.slog2 >= 1 && lay.slog2 < 5) {
+  if (op0 == 0 && op1 == V && width >= kRingMinCols && cols <= kMaxCols && lay.slog2 >= 1 && lay.slog2 < 5) {
     const int64_t tiles = (V + kRingOps - 1) / kRingOps;
     const dim3 grid((unsigned)std::min<int64_t>(tiles, std::max<int64_t>(1, 152 / cols)), (unsigned)cols);
     const cudaError_t e = cudaFuncSetAttribute(readback_all_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmem);
@@ -710,11 +711,13 @@ cudaError_t launch_readback(const int32_t *ext2int, const int32_t *int2ext, int6
     readback_all_kernel<<<grid, 256, kRingSmem, st>>>(int2ext, V, s0, s1, width, lay, f, d, cidx, lay_c, cd, start, finish);
     return cudaGetLastError();
   }
-  if (s1 - s0 >= kReadCols && lay.slog2 < 5) {
-    const int32_t first = s0 & ~(kReadCols - 1);
-    const int64_t cols = (s1 - first + kReadCols - 1) / kReadCols, tiles = (op1 - op0 + kTileOps - 1) / kTileOps;
+  // (about two million scenarios at most: with that many an op's row is long enough for any kernel)
+  const int32_t first = s0 & ~(kReadCols - 1);
+  const int64_t tile_cols = ((int64_t)s1 - first + kReadCols - 1) / kReadCols;
+  if (s1 - s0 >= kReadCols && lay.slog2 < 5 && tile_cols <= kMaxCols) {
+    const int64_t tiles = (op1 - op0 + kTileOps - 1) / kTileOps;
     // one wave of blocks: 4 of 256 threads on an SM
-    const dim3 grid((unsigned)std::min<int64_t>(tiles, std::max<int64_t>(1, 152 * 4 / cols)), (unsigned)cols);
+    const dim3 grid((unsigned)std::min<int64_t>(tiles, std::max<int64_t>(1, 152 * 4 / tile_cols)), (unsigned)tile_cols);
     readback_tile_kernel<<<grid, 256, 0, st>>>(ext2int, op0, op1, s0, s1, lay, f, d, cidx, lay_c, cd, start, finish);
     return cudaGetLastError();
   }

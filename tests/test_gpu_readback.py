@@ -7,6 +7,7 @@ import pytest
 import oracle
 from paper_2412_12487_gb300 import Echo, EchoError
 from paper_2412_12487_gb300 import workloads as W
+from tests import smallgraphs as SG
 
 pytestmark = pytest.mark.gpu
 
@@ -71,3 +72,20 @@ def test_sums_still_refuse_what_could_overflow():
                 e.estimate_collectives()
                 e.compose()
                 assert np.array_equal(e.read_makespan(), oracle.compose(g, sc).makespan)
+
+
+@pytest.mark.parametrize("S", [32 * 65535, 32 * 65535 + 1])
+def test_more_scenarios_than_the_tiles_have_columns(S):
+    g = SG.graph_from_lists(1, 2, [{"kind": W.KIND_COMPUTE, "kclass": 0, "preds": []} for _ in range(3)], {(0, 0): [0, 1, 2]}, [[0]],
+                            gpus_per_node=1)
+    sc = SG.random_scenarios(np.random.default_rng(1), g, S, max_dur=1000)
+    want = np.cumsum(sc.dur, axis=0)
+    with Echo(0) as e:
+        e.load_graph(g)
+        e.load_scenarios(sc)
+        e.estimate_collectives()
+        e.compose(refine_passes=0)
+        for op0, op1 in ((0, 2), (0, 3)):  # tiles in the caller's order; every op, S past the end of the tiles' columns
+            st, fn = e.read_times(op0, op1)
+            assert np.array_equal(fn, want[op0:op1]) and np.array_equal(st, (want - sc.dur)[op0:op1])
+        assert np.array_equal(e.read_makespan(), want[-1])
