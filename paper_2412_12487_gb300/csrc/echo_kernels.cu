@@ -23,11 +23,12 @@ constexpr int kRing = 0, kTree = 1;
 
 // ceil(a / b), a >= 0, b > 0.  Quotients of the estimator (chunk rounds) are small, and a
 // 64-bit division takes about 100 instructions: an estimate in fp32 is off by at most
-// q * 2^-21 + 1 < 2 below 2^20, which the remainder puts right.
+// q * 2^-21 + 1 < 2 below 2^20, which the remainder puts right.  (b is a product and may
+// have wrapped below 0, like a sum n: both take the division.)
 __device__ __forceinline__ int64_t cdiv64(int64_t a, int64_t b) {
   const int64_t n = a + b - 1;
   const float q0 = __fdividef((float)n, (float)b);
-  if (!(q0 < 1048576.0f) || n < 0 || b >= (1ll << 40)) return n / b;
+  if (!(q0 < 1048576.0f) || n < 0 || (uint64_t)b >= (1ull << 40)) return n / b;
   int32_t q = (int32_t)q0;
   int64_t r = n - (int64_t)q * b;
   if (r < 0) { --q; r += b; }

@@ -78,6 +78,20 @@ def test_queries_equal_the_oracle(forms, n, table, copies, monkeypatch):
         assert np.array_equal(t.cpu().numpy(), want)
 
 
+def test_a_chunk_times_the_ranks_beyond_64_bits():
+    # 12 ranks with chunks of 2^60 bytes: every message is one round, also where the 64-bit product is negative
+    size, N = (1 << 62) + (1 << 61), 12
+    prm = [7.0, 3.0, 11.0, 5.0, 13.0, 0.25]
+    host = [np.array([1], np.uint8), np.array([0], np.uint8), np.array([size]), np.array([N], np.int32), np.array([1], np.int32)]
+    host += [np.array([x]) for x in prm]
+    most, chunk = np.array([(1 << 63) - 1]), np.array([1 << 60])
+    out = np.zeros(1)
+    with E.Echo(0) as e:
+        d = E.CCQueryDesc(1, *[h.ctypes.data for h in host], 1, most.ctypes.data, chunk.ctypes.data)
+        assert e.lib.echo_cc_query(e.h, C.byref(d), C.c_void_p(out.ctypes.data)) == 0
+    assert out[0] == 7.0 + (N - 1) * (11.0 + float(size) / N / 3.0)
+
+
 def test_parameters_uploaded_or_read_in_place(monkeypatch):
     c = W.GPTConfig(**{**W.config("tiny").__dict__, "fixed_scenario": False})
     g = W.build_gpt_graph(c)
