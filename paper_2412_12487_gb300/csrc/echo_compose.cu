@@ -202,8 +202,8 @@ __device__ __noinline__ bool segment_ok(const StagedArgs &a, uint32_t first, uin
 // the record ring at word `ro`; its rows are i0 + header.z ... (global rows), held in
 // the duration ring of RR rows (a power of two) from ring row dpos0 + header.z on
 // (wrapping).  Thread `sub` handles segments sub, sub + step, ... for scenario
-// lanes j0 .. j0+LANES-1; the segments of a level come heaviest first, so a warp's
-// lanes hold segments of similar weight.  Every input of a head is the tail of an earlier segment: the
+// lanes j0 .. j0+LANES-1; the segments of a level come longest first, so a warp's
+// lanes hold segments of similar length.  Every input of a head is the tail of an earlier segment: the
 // recent ones are read from the value ring (entries are byte offsets of their
 // slots), older ones from global memory (entries are node ids).  Inputs and
 // durations are loaded four at a time so that their latencies overlap.  This
@@ -300,8 +300,12 @@ __device__ __forceinline__ void compose_segments(const StagedArgs &a, uint32_t r
   }
 }
 
-// Staged compose (all threads copy and compose).  Shared memory holds the
-// per-scenario makespans, the extents of the last 16 copy groups, two metadata
+// Staged compose (all threads copy and compose): for graphs whose levelled plan does not fit
+// shared memory.  What bounds it is the serial work of a level, copies and all.  After the
+// first composition a candidate's duration is copied from its row of the validator's compact
+// matrix.  (A full matrix of all durations, made by a copy and a scatter before each
+// composition, cost 11.5 of the 38.5 ms of 1024 ranks with 32 layers x 1024, and 12.6 GB;
+// the lookups of the rows cost 1.3.)  Shared memory holds the per-scenario makespans, the extents of the last 16 copy groups, two metadata
 // buffers (kMetaChunk segment levels each), the frontier, a value ring with the
 // finish times of the tails of the most recent 2^vlog2 segments (read by near
 // predecessors), a ring of duration rows and a ring of record words.  Before
@@ -339,17 +343,37 @@ compose_staged_kernel(StagedArgs a) {
   // this block's rows are contiguous: element e of the block lands in ring element
   // e mod (RR*SIGMA), and a 16-byte piece never straddles the ring's end
   const int64_t *durb = a.dur + ((int64_t)blockIdx.x * a.pitch) * SIGMA;
+  const int64_t *cdurb = a.cdur ? a.cdur + ((int64_t)blockIdx.x * a.c_pitch) * SIGMA : nullptr;
   const uint32_t emask = RR * SIGMA - 1;
   uint32_t rows_done = 0, words_done = 0;
+  auto copy = [&](uint32_t e, const int64_t *src) {  // LANES elements into the ring
+    if constexpr (LANES == 2)
+      cp_async16(dr + (e & emask), src);
+    else
+      cp_async8(dr + (e & emask), src);
+  };
   auto issue_to = [&](uint32_t row_lim, uint32_t word_lim) {  // copy rows and words up to the limits
-    if constexpr (SIGMA % 2 == 0) {
-      const uint32_t e0 = rows_done * SIGMA, n16 = (row_lim - rows_done) * (SIGMA / 2);
-      for (uint32_t t = tid; t < n16; t += blockDim.x) {
-        const uint32_t e = e0 + 2 * t;
-        cp_async16(dr + (e & emask), durb + e);
-      }
+    const uint32_t end = row_lim * TPN;  // pieces of LANES elements
+    if (!cdurb) {
+      for (uint32_t t = rows_done * TPN + tid; t < end; t += THREADS) copy(LANES * t, durb + LANES * t);
     } else {
-      for (uint32_t e = rows_done + tid; e < row_lim; e += blockDim.x) cp_async8(dr + (e & emask), durb + e);
+      // a candidate's row comes from the validator's matrix; kLook rows are looked up together
+      constexpr int kLook = 8;
+      for (uint32_t t0 = rows_done * TPN + tid; t0 < end; t0 += kLook * THREADS) {
+        int32_t ci[kLook];
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) ci[u] = t0 + u * THREADS < end ? __ldg(a.cidx + (t0 + u * THREADS) / TPN) : -1;
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) {
+          const uint32_t t = t0 + u * THREADS, e = LANES * t;
+          if (t >= end) break;
+          if (a.dbg && ci[u] >= 0 && !in_range(ci[u], a.c_rows)) {  // debug bounds
+            atomicCAS(a.status, 0, (int32_t)kDevBounds);
+            ci[u] = -1;
+          }
+          copy(e, ci[u] >= 0 ? cdurb + (int64_t)ci[u] * SIGMA + e % SIGMA : durb + e);
+        }
+      }
     }
     for (uint32_t t = words_done + tid * 4; t < word_lim; t += blockDim.x * 4)
       cp_async16(&rr[t & rmask], &a.recs[t]);

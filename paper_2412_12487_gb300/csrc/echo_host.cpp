@@ -1532,7 +1532,7 @@ struct echo_ctx {
   void *raw = nullptr;
   int64_t *dur = nullptr, *f[2] = {nullptr, nullptr}, *mk = nullptr, *cc_dur = nullptr;
   int64_t *gfrontier = nullptr;
-  int64_t *deff = nullptr;                // full validator durations, for kernels without a candidate ring
+  int64_t *deff = nullptr;                // full validator durations, for the direct composer
   int64_t *cd[2] = {nullptr, nullptr};    // candidates' durations of the validator's passes (compact)
   echo::MatLayout lay_c{0, 0};            // [n_cand][S] compact layout
   size_t cd_elems = 0;                    // elements of each compact matrix
@@ -2074,7 +2074,7 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
     CK(cudaMemsetAsync(c->dur, 0, VS * sizeof(int64_t), c->stream), "memset");
     CK(cudaMemsetAsync(c->cd[0], 0, CS * sizeof(int64_t), c->stream), "memset");
     c->cd[1] = nullptr;   // second compact buffer: allocated when refine_passes > 1
-    c->deff = nullptr;    // allocated when a kernel without a candidate ring composes a second pass
+    c->deff = nullptr;    // allocated when the direct kernel composes a second pass
     // launch shape of the staged kernels (threads and blocks per SM may be overridden
     // for tuning: ECHO_STAGED_THREADS, ECHO_BLOCKS_PER_SM)
     int optin = 0, per_sm = 0;
@@ -2216,9 +2216,10 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
   const char *dbg_env = std::getenv("ECHO_DEBUG_BOUNDS");
   const int32_t dbg = (opts && opts->debug_bounds) || (dbg_env && std::atoi(dbg_env) != 0) ? 1 : 0;
   const GraphBuild &B = c->gb;
-  // the levelled and dataflow composers read the validator's durations of the
-  // candidates (compact rows); the others compose from a full matrix built for them
-  const bool ring = c->use_df || c->lplan.ok;
+  // the composers read the validator's durations of the candidates (compact rows), all but
+  // the direct one, which composes from a full matrix built for it
+  const bool staged = c->plan.ok && c->kernel_choice != 1;
+  const bool ring = c->use_df || c->lplan.ok || staged;
   if (refine > 1 && !c->cd[1]) {
     if ((rc = dalloc(c, c->scen_allocs, &c->cd[1], c->cd_elems))) return rc;
     CK(cudaMemsetAsync(c->cd[1], 0, c->cd_elems * sizeof(int64_t), c->stream), "memset");
@@ -2346,7 +2347,7 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
       a.n_recs_kept = (c->lplan.ends - c->lplan.recs_kept) / 4;
       return timed(c, name, [&] { return echo::launch_compose_levels(a, c->sigma, c->stream); });
     }
-    if (c->plan.ok && c->kernel_choice != 1) {
+    if (staged) {
       echo::StagedArgs a{};
       a.S = c->S;
       a.L = (int32_t)c->steps.L;
@@ -2359,12 +2360,16 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
       a.meta = c->d_meta;
       a.recs = c->d_recs;
       a.dur = d;
+      a.cdur = B.n_cand ? cdur : nullptr;
+      a.cidx = c->cidx;
+      a.c_pitch = c->lay_c.V;
+      a.c_rows = B.n_cand;
       a.f = f;
       a.makespan = c->mk;
       a.status = c->status;
       a.store_all = final_pass;
       a.dbg = dbg;
-      return timed(c, name, [&] { return echo::launch_compose_staged(a, c->sigma, c->plan, c->stream); });
+      return timed(c, "compose_staged", [&] { return echo::launch_compose_staged(a, c->sigma, c->plan, c->stream); });
     }
     echo::ComposeArgs a{};
     a.V = B.V;

@@ -98,6 +98,9 @@ struct StagedArgs {
   const uint32_t *meta;          // [4*(L+1)]: record word offset, first node, first segment, 0
   const uint32_t *recs;          // record blocks
   const int64_t *dur;            // durations (MatLayout)
+  const int64_t *cdur;           // candidates' durations (compact), or null: the original ones
+  const int32_t *cidx;           // [n_rows] compact row of a candidate, -1 otherwise
+  int64_t c_pitch, c_rows;       // rows of a scenario block of cdur, candidates
   int64_t *f;                    // finish times (MatLayout, out)
   int64_t *makespan;             // [S] (out)
   int32_t *status;               // device status word

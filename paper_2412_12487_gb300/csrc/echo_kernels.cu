@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(256) readback_all_kernel(const int32_t *__rest
   }
 }
 
-// Full validator durations for the kernels without a candidate ring: the
+// Full validator durations for the direct composer: the
 // candidates' rows of the compact cd into dst (which holds the original durations).
 __global__ void scatter_candidates_kernel(const int32_t *__restrict__ cand_node, int64_t n_cand, int32_t S,
                                           MatLayout lay, MatLayout lay_c, const int64_t *__restrict__ cd,

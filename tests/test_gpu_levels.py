@@ -80,3 +80,29 @@ def test_debug_bounds_of_every_block_width(sigma, monkeypatch):
                 st, fn = e.read_times()
                 got = dict(start=st, finish=fn, makespan=e.read_makespan(), cc=e.read_cc(), ov=e.read_overlap())
                 assert_same(got, oracle.compose(g, sc, refine_passes=refine, overlap_model=model, comm_interval=interval), g, refine)
+
+
+@pytest.mark.parametrize("ranks,S,kernel", [(1000, 70, None), (1000, 17, "pipelined"), (1000, 17, "staged"), (40, 5, "staged")])
+def test_without_a_levelled_plan(ranks, S, kernel, monkeypatch):
+    """More live tails than half of a block's shared memory holds (1000 in blocks of 16): the staged composer runs, and
+    reads the validator's durations where they are, without a full matrix made of them."""
+    monkeypatch.setenv("ECHO_SIGMA", "16" if ranks == 1000 else "1")
+    if kernel:
+        monkeypatch.setenv("ECHO_COMPOSE_KERNEL", kernel)
+    g = _joins(ranks, [1, 2, 5, 65] if ranks == 40 else [1, 2, 5])
+    sc = SG.random_scenarios(np.random.default_rng(S), g, S, max_dur=20_000)
+    with Echo(0) as e:
+        e.set_profiling(True)
+        for refine, model, interval in ((0, 0, 0), (1, 0, 0), (2, 1, 1), (3, 0, 0)):
+            for debug in (False, True):
+                e.load_graph(g)
+                e.load_scenarios(sc)
+                e.estimate_collectives()
+                e.compose(refine_passes=refine, overlap_model=model, comm_interval=interval, debug_bounds=debug)
+                st, fn = e.read_times()
+                got = dict(start=st, finish=fn, makespan=e.read_makespan(), cc=e.read_cc(), ov=e.read_overlap())
+                want = oracle.compose(g, sc, refine_passes=refine, overlap_model=model, comm_interval=interval)
+                assert_same(got, want, g, refine)
+                ran = e.read_profile()
+                assert ran["compose_staged"][0] == refine + 1
+                assert not {"scatter_candidates", "compose", "compose_adjusted", "compose_direct"} & set(ran)
