@@ -312,8 +312,8 @@ typedef struct {
   int64_t n_ops_composed;    /* ops of the graph being composed                       */
   int32_t n_ranks, n_streams, sigma; /* sigma: scenarios per thread block of the composer;
                                         32: the dataflow composer (a warp per rank and 32
-                                        scenarios), chosen for graphs with many levels and
-                                        few scenarios */
+                                        scenarios).  The library runs the composer, and the
+                                        width, with the smallest estimate of a step's time */
   int32_t replicas_folded;
   int64_t n_validator_comm_entries; /* (comm op, member rank) pairs the validator's cursors
                                        visit: those that can overlap a compute op of the rank */

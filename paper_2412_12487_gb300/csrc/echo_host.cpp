@@ -99,6 +99,7 @@ struct GraphBuild {
   std::vector<int64_t> df_off;
   std::vector<uint32_t> df_rec, df_opnd;
   int64_t df_slots = 0, df_exports = 0;
+  int64_t df_joins = 0;  // most joins with ranks of other blocks in one rank's program
   int32_t df_wpb = 1;  // warps per block: a block holds df_wpb consecutive ranks (for block joins)
   bool stageable = true;              // every head has < 2^16 inputs
 };
@@ -314,7 +315,7 @@ void build_dataflow(GraphBuild &b) {
   // each timeline and the previous op are kept
   for (int32_t r = 0; r < R; ++r) b.df_off[r + 1] = b.df_off[r] + (b.q_off[(int64_t)(r + 1) * NS] - b.q_off[(int64_t)r * NS]);
   b.df_rec.assign((size_t)b.df_off[R] * 8, 0u);
-  std::vector<int64_t> cnt(R, 0);
+  std::vector<int64_t> cnt(R, 0), joins(R, 0);
   std::vector<int32_t> last((size_t)R * NS, -1), prev(R, -1);
   std::vector<int8_t> prev_tl(R, 0);
   std::vector<uint32_t> extra;
@@ -350,6 +351,7 @@ void build_dataflow(GraphBuild &b) {
         use_prev = true;
         regs &= ~(1u << prev_tl[r]);
       }
+      joins[r] += comm && nm > 1 && !(slot[v] & echo::kDfBlockJoin);
       const bool two_hop = comm && nm > (int64_t)echo::kDfDirectMembers;
       const bool publish = exp_id[v] >= 0 && (!comm || me == 0);
       if (extra.size() > 0xFF || nm > 0xFFFF || b.df_opnd.size() + extra.size() >= (size_t)UINT32_MAX) return;
@@ -374,6 +376,7 @@ void build_dataflow(GraphBuild &b) {
   if (b.df_slots >= (int64_t)echo::kDfBlockJoin) return;
   for (uint32_t n : bseq)
     if (n >= echo::kDfBlockJoin) return;
+  b.df_joins = *std::max_element(joins.begin(), joins.end());
   if (b.df_rec.empty()) b.df_rec.assign(8, 0);
   if (b.df_opnd.empty()) b.df_opnd.push_back(0);
   b.df_ok = true;
@@ -1266,7 +1269,8 @@ struct LevelPlan {
   int64_t heads = 0, recs_all = 0, recs_kept = 0, ends = 0;
 };
 
-LevelPlan plan_levels(const GraphBuild &b, int sigma, size_t smem_cap) {
+// fill: also write what the device reads (else only whether a plan fits, and its steps).
+LevelPlan plan_levels(const GraphBuild &b, int sigma, size_t smem_cap, bool fill = true) {
   LevelPlan P;
   if (!b.stageable || b.n_seg == 0) return P;
   const int64_t row = (int64_t)sigma * 8, pad = sigma == 1 ? 1 : 0;
@@ -1369,6 +1373,10 @@ LevelPlan plan_levels(const GraphBuild &b, int sigma, size_t smem_cap) {
   }
   if (!fits) return P;
   P.L = (int64_t)parts.size();
+  if (!fill) {
+    P.ok = true;
+    return P;
+  }
   P.ring_bytes = (uint32_t)ring;
   P.smem_bytes = (uint32_t)(P.ring_at + ring + echo::kLvSlackBytes);
   const uint32_t zero = place_of_slot(0), nobody = place_of_slot(1);
@@ -1487,9 +1495,15 @@ struct DevArr {
 
 }  // namespace
 
+// The composer of a batch (choose_composer).
+struct Choice {
+  bool df = false, levels = false;  // neither: the staged composer, or the direct one
+  int sigma = 1;
+};
+
 struct echo_ctx {
   int device = 0;
-  int sms = 0;
+  int sms = 0, smem_block = 0, smem_sm = 0;  // of the device: SMs, shared memory of a block and of an SM
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   std::string err;
@@ -1551,6 +1565,8 @@ struct echo_ctx {
   int kernel_choice = 0;            // 0 automatic, 1 direct, 2 staged, 3 levelled, 4 dataflow (tuning and tests)
   // dataflow composer
   bool use_df = false;
+  Choice choice;
+  int width = 0;  // the blocks that S alone asks for
   int64_t *df_off = nullptr;
   uint32_t *df_rec = nullptr, *df_opnd = nullptr;
   uint64_t *df_part = nullptr, *df_xval = nullptr;
@@ -1662,15 +1678,92 @@ int check_ctx(echo_ctx *c) {
   return ECHO_OK;
 }
 
+int forced_sigma() {  // tuning override: 1, 2, 4, 8 or 16 (0: none)
+  const char *e = std::getenv("ECHO_SIGMA");
+  const int v = e ? std::atoi(e) : 0;
+  return v == 1 || v == 2 || v == 4 || v == 8 || v == 16 ? v : 0;
+}
+
+// Shared memory of a levelled block, of a staged one (ECHO_BLOCKS_PER_SM: tuning).
+size_t level_smem(const echo_ctx *c) { return (size_t)std::max(c->smem_block - 1024, 0); }
+size_t staged_smem(const echo_ctx *c) {
+  const char *e = std::getenv("ECHO_BLOCKS_PER_SM");
+  const int blocks = e ? std::max(1, std::atoi(e)) : 1;
+  return std::min(level_smem(c), (size_t)(c->smem_sm / blocks) - 1024);
+}
+
 int pick_sigma(int32_t S, int sms) {
-  if (const char *e = std::getenv("ECHO_SIGMA")) {  // tuning override: 1, 2, 4, 8 or 16
-    int v = std::atoi(e);
-    if (v == 1 || v == 2 || v == 4 || v == 8 || v == 16) return v;
-  }
+  if (const int v = forced_sigma()) return v;
   int want = (S + sms - 1) / std::max(sms, 1);
   int s = 1;
   while (s < want && s < 16) s <<= 1;
   return s;
+}
+
+// The staged composer's steps and plan for blocks of `sigma`: the widest steps whose rings fit.
+echo::StagedPlan plan_steps(const GraphBuild &B, int sigma, size_t smem_cap, Steps &steps) {
+  echo::StagedPlan plan;
+  for (int64_t step_cap = kStepNodes;; step_cap /= 2) {
+    steps = make_steps(B, step_cap);
+    plan = plan_staged(B, steps, sigma, smem_cap);
+    if (plan.ok || step_cap <= 2 * echo::kMaxSegment) return plan;
+  }
+}
+
+// The composer and block width of a batch of S scenarios: of those that can run, the one with
+// the smallest estimate of a step (two compositions and the validator between them).
+// Estimates in us, KB: a block's duration rows; pairs: candidates x scenarios.
+//   levelled   0.3 a step of its plan + 0.03 a KB, each composition and wave of blocks.
+//              Graphs of 8 to 1024 ranks, blocks of 1 to 16, estimate against the final
+//              composition: GPT-175B x 152, 250, 1024 1177 / 951, 1445 / 1196, 3442 / 3100;
+//              1024 ranks (32 layers) x 152, 200 1247 / 1157, 1990 / 2064, 512 ranks
+//              interleaved x 152 637 / 614, x 400 1567 / 1931; GPT-1.3B x 256 243 / 178.
+//   dataflow   0.155 a level of ops and 2.7 a join with ranks of other blocks (the schedule's
+//              longest path and what its warps wait), 2.5% more for each warp on an SM past
+//              four: 1024 ranks x 64 918 / 1046, 512 interleaved x 64 725 / 673, GPT-175B x 1
+//              2766 / 3056, GPT-1.3B x 608 624 / 506, 96 interleaved x 608 891 / 919.
+//   staged     0.85 a level + 0.052 a KB (blocks of 8 and 16), against the mean of both
+//              compositions: 512 ranks interleaved x 1024 2917 / 3647, 512 of data parallelism
+//              x 1024 2700 / 3100, 256 interleaved x 1280 2918 / 2933.
+//   validator  0.020 to 0.0075 a thousand pairs: narrow blocks take more, as the teams of a
+//              warp move their cursors one after the other.
+// Where a levelled plan does not fit at the batch's own width it often does at half of it:
+// 512 ranks of data parallelism x 1024 take 5.5 ms a step so, staged 7.1; but with many
+// candidates the wider blocks are the cheaper ones (512 interleaved: 16.1 against 13.8).
+Choice choose_composer(const echo_ctx *c, const GraphBuild &B, int32_t S, int width) {
+  Choice best;
+  best.sigma = width;
+  if (c->kernel_choice == 1 || c->kernel_choice == 2) return best;
+  auto waves = [&](int s) { return (double)(((S + s - 1) / s + c->sms - 1) / std::max(c->sms, 1)); };
+  auto kb = [&](int s) { return (double)B.V * s * 8 / 1024; };
+  auto validator = [&](int s) {
+    const double ns[6] = {0.020, 0.0125, 0.0105, 0.0085, 0.0080, 0.0075};
+    return (double)B.n_cand * S * 1e-3 * ns[__builtin_ctz(s)];
+  };
+  double best_us = 2 * waves(width) * (0.85 * B.Ls + 0.052 * kb(width)) + validator(width);
+  for (int s = width; s >= 1 && c->kernel_choice != 4; s /= 2) {
+    if (s < width && forced_sigma()) break;
+    const LevelPlan P = plan_levels(B, s, level_smem(c), false);
+    if (!P.ok) continue;
+    const double us = 2 * waves(s) * (0.3 * P.L + 0.03 * kb(s)) + validator(s);
+    Steps steps;
+    if (s < width && us >= best_us && c->kernel_choice == 0 && plan_steps(B, width, staged_smem(c), steps).ok) break;
+    best.levels = true;
+    best.sigma = s;
+    best_us = us;
+    break;
+  }
+  const int32_t n_groups = (S + 31) / 32;
+  if (B.df_ok && c->kernel_choice != 3 && echo::dataflow_fits((int64_t)B.R * n_groups, B.NS, B.df_wpb, c->device)) {
+    const double warps = (double)B.R * n_groups / std::max(c->sms, 1);
+    const double us = 2 * (0.155 * B.L + 2.7 * B.df_joins) * (1 + 0.025 * std::max(0.0, warps - 4)) + validator(32);
+    if (c->kernel_choice == 4 || us < best_us) {
+      best.df = true;
+      best.levels = false;
+      best.sigma = 32;
+    }
+  }
+  return best;
 }
 
 // Waits for the stream's work and reads words [first, end) of `small` into h_small;
@@ -1818,7 +1911,9 @@ int echo_create(echo_ctx **out, int device, void *cuda_stream) {
   if (!c) return ECHO_E_OOM;
   c->device = device;
   if (cudaSetDevice(device) != cudaSuccess ||
-      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->smem_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device) != cudaSuccess) {
     delete c;
     return ECHO_E_CUDA;
   }
@@ -1997,33 +2092,13 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
     if ((rc = activate_fold(c, h_flag == 0))) return rc;
   }
   const int64_t V = B.V;
-  // The dataflow composer (rows of 32 scenarios, a warp per rank) is serial in the length
-  // of the longest rank program, the levelled one in its number of steps.  Measured on
-  // GB300: a program entry costs about 0.22 us while at most 8 warps share an SM, and
-  // proportionally more beyond; a levelled step about 0.22 us and 0.026 us per KB of its
-  // rows (GPT-1.3B x 1, 256: 0.24 and 0.29 us with 2 and 4 KB a step; GPT-175B x 250, 1024:
-  // 0.37 and 0.65 us with 6 and 17 KB).  The cheaper estimate wins (when every warp can be
-  // resident).
   const int32_t n_groups = (S + 31) / 32;
-  bool use_df = false;
-  if (B.df_ok && (c->kernel_choice == 0 || c->kernel_choice == 4) &&
-      echo::dataflow_fits((int64_t)B.R * n_groups, B.NS, B.df_wpb, c->device)) {
-    int64_t longest = 0;
-    for (int32_t r = 0; r < B.R; ++r) longest = std::max(longest, B.df_off[r + 1] - B.df_off[r]);
-    const double warps_per_sm = (double)B.R * n_groups / std::max(c->sms, 1);
-    const double df_us = (double)longest * 0.22 * std::max(1.0, warps_per_sm / 8.0);
-    // (steps of at most 128 segments or a fifth of the ring; rows of all blocks' scenarios)
-    const int lev_sigma = pick_sigma(S, c->sms);
-    double steps = 0;
-    for (int64_t l = 0; l < B.Ls; ++l) {
-      const int64_t segs = B.seg_lvl_off[l + 1] - B.seg_lvl_off[l];
-      const int64_t rows = B.seg_node_off[B.seg_lvl_off[l + 1]] - B.seg_node_off[B.seg_lvl_off[l]];
-      steps += (double)std::max<int64_t>({1, (segs + 127) / 128, rows * lev_sigma * 8 / 40000});
-    }
-    const double lev_us = steps * 0.22 + (double)B.V * lev_sigma * 8 / 1024 * 0.026;
-    use_df = c->kernel_choice == 4 || df_us < lev_us;
-  }
-  const int sigma = use_df ? 32 : pick_sigma(S, c->sms);
+  const int width = pick_sigma(S, c->sms);
+  if (c->scen_vs == 0 || c->S != S || c->width != width)  // (else it is the choice of the last batch)
+    c->choice = choose_composer(c, B, S, width);
+  c->width = width;
+  const bool use_df = c->choice.df;
+  const int sigma = c->choice.sigma;
   int slog2 = 0;
   while ((1 << slog2) < sigma) ++slog2;
   // [op][scenario] matrices are stored in scenario blocks of sigma (the last padded)
@@ -2075,37 +2150,23 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
     CK(cudaMemsetAsync(c->cd[0], 0, CS * sizeof(int64_t), c->stream), "memset");
     c->cd[1] = nullptr;   // second compact buffer: allocated when refine_passes > 1
     c->deff = nullptr;    // allocated when the direct kernel composes a second pass
-    // launch shape of the staged kernels (threads and blocks per SM may be overridden
-    // for tuning: ECHO_STAGED_THREADS, ECHO_BLOCKS_PER_SM)
-    int optin = 0, per_sm = 0;
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device);
-    int threads = sigma == 16 ? 1024 : sigma == 8 ? 512 : sigma == 4 ? 256 : 512;
-    int bps = 1;
-    if (const char *e = std::getenv("ECHO_STAGED_THREADS")) threads = std::atoi(e);
-    if (const char *e = std::getenv("ECHO_BLOCKS_PER_SM")) bps = std::max(1, std::atoi(e));
-    const size_t cap = std::min((size_t)std::max(optin - 1024, 0), (size_t)(per_sm / bps) - 1024);
     c->lplan = LevelPlan{};
     c->plan = echo::StagedPlan{};
-    if (!use_df && (c->kernel_choice == 0 || c->kernel_choice == 3)) {
+    if (c->choice.levels) {
       LevelPlan &P = c->lplan;
-      P = plan_levels(B, sigma, (size_t)std::max(optin - 1024, 0));
-      if (P.ok) {
-        if ((rc = upload(c, o, &c->d_meta, P.words))) {
-          free_all(c->scen_allocs);
-          return rc;
-        }
-        CK(cudaStreamSynchronize(c->stream), "plan upload");
-        P.words = std::vector<uint32_t>();
+      P = plan_levels(B, sigma, level_smem(c));
+      if ((rc = upload(c, o, &c->d_meta, P.words))) {
+        free_all(c->scen_allocs);
+        return rc;
       }
+      CK(cudaStreamSynchronize(c->stream), "plan upload");
+      P.words = std::vector<uint32_t>();
+    } else if (!use_df && c->kernel_choice != 1) {
+      c->plan = plan_steps(B, sigma, staged_smem(c), c->steps);
     }
-    // the staged kernel: the widest steps whose rings fit
-    for (int64_t step_cap = kStepNodes; !use_df && !c->lplan.ok && c->kernel_choice != 1; step_cap /= 2) {
-      c->steps = make_steps(B, step_cap);
-      c->plan = plan_staged(B, c->steps, sigma, cap);
-      if (c->plan.ok || step_cap <= 2 * echo::kMaxSegment) break;
-    }
-    c->plan.threads = threads;
+    // (threads of a staged block; may be overridden for tuning)
+    c->plan.threads = sigma == 16 ? 1024 : sigma == 8 ? 512 : sigma == 4 ? 256 : 512;
+    if (const char *e = std::getenv("ECHO_STAGED_THREADS")) c->plan.threads = std::atoi(e);
     if (c->plan.ok) {
       std::vector<uint32_t> recs, meta;
       build_records(B, c->steps, sigma, c->plan.vring_log2, recs, meta);

@@ -106,3 +106,27 @@ def test_without_a_levelled_plan(ranks, S, kernel, monkeypatch):
                 ran = e.read_profile()
                 assert ran["compose_staged"][0] == refine + 1
                 assert not {"scatter_candidates", "compose", "compose_adjusted", "compose_direct"} & set(ran)
+
+
+@pytest.mark.parametrize("lengths,S,sigma,ran", [([30], 1217, 8, "compose"), ([1, 2, 5], 1217, 16, "compose_staged"),
+                                                 ([30], 5, 32, "compose"), ([1, 2, 5], 5, 1, "compose"),
+                                                 ([30], 200, 2, "compose")])
+def test_choice_among_composers_that_exist(lengths, S, sigma, ran):
+    """950 ranks: 1217 scenarios ask for blocks of 16, in which the tails do not fit.  Long chains take the levelled
+    composer in blocks of 8, short ones the staged one; few scenarios the dataflow composer where a rank's chain is long
+    beside its joins; narrower blocks have a levelled plan of their own."""
+    g = _joins(950, lengths)
+    sc = SG.random_scenarios(np.random.default_rng(S), g, S, max_dur=20_000)
+    with Echo(0) as e:
+        e.set_profiling(True)
+        e.load_graph(g)
+        for _ in range(2):  # (a second batch keeps the first one's choice)
+            e.load_scenarios(sc)
+            e.estimate_collectives()
+            e.read_profile()
+            e.compose()
+            st, fn = e.read_times()
+            got = dict(start=st, finish=fn, makespan=e.read_makespan(), cc=e.read_cc(), ov=e.read_overlap())
+            assert e.info()["sigma"] == sigma
+            assert [k for k in e.read_profile() if k.startswith("compose")][0] == ran
+            assert_same(got, oracle.compose(g, sc, threads=8), g)
