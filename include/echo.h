@@ -254,8 +254,9 @@ int echo_compose(echo_ctx *ctx, const echo_compose_opts *opts);
  * (op1-op0)*(s1-s0) int64 each, row-major [op][s - s0]: host memory (pageable or
  * pinned) or device memory of the context's device.  Either may be NULL.  A range
  * outside [0, n_ops) x [0, n_scen) or an empty scenario range with ops:
- * ECHO_E_INVALID_ARG.  Large ranges are read back in chunks through a staging
- * buffer of the context. */
+ * ECHO_E_INVALID_ARG.  Aligned buffers in the device's own memory are written
+ * directly; anything else is read back in chunks through a staging buffer of the
+ * context. */
 int echo_read_times(echo_ctx *ctx, int64_t op0, int64_t op1, int32_t s0, int32_t s1, int64_t *start,
                     int64_t *finish);
 /* Step time per scenario: the largest finish time (0 for an empty graph). [S] */

@@ -1528,7 +1528,7 @@ struct echo_ctx {
   uint8_t *cand_flag = nullptr;
   int32_t *nq = nullptr, *dp = nullptr, *q_ops = nullptr, *int2ext = nullptr, *ext2int = nullptr;
   int32_t *node_sig = nullptr, *comm_node = nullptr, *comm_sig = nullptr, *sig_count = nullptr;
-  uint8_t *kcl = nullptr, *local = nullptr;
+  uint8_t *local = nullptr;
   CcSig *sigs = nullptr;
   // [S] sums, [S] comm_sum, a status word, [S] makespans lie one behind the other in
   // `small`, so that each call reads its status and results back with one copy
@@ -1845,7 +1845,7 @@ int upload_graph(echo_ctx *c) {
       (rc = upload(c, o, &c->q_ops, B.q_ops_int)) || (rc = upload(c, o, &c->int2ext, B.int2ext)) ||
       (rc = upload(c, o, &c->ext2int, B.ext2int)) || (rc = upload(c, o, &c->node_sig, B.node_sig)) ||
       (rc = upload(c, o, &c->comm_node, B.comm_node)) || (rc = upload(c, o, &c->comm_sig, B.comm_sig)) ||
-      (rc = upload(c, o, &c->sig_count, B.sig_count)) || (rc = upload(c, o, &c->kcl, B.kcl)) ||
+      (rc = upload(c, o, &c->sig_count, B.sig_count)) ||
       (rc = upload(c, o, &c->local, B.local)) ||
       (rc = upload(c, o, &c->sigs, B.sigs)) ||
       (B.df_ok && ((rc = upload(c, o, &c->df_off, B.df_off)) || (rc = upload(c, o, &c->df_rec, B.df_rec)) ||
@@ -1937,7 +1937,7 @@ int echo_create(echo_ctx **out, int device, void *cuda_stream) {
                       cudaSuccess && in_place && !std::getenv("ECHO_TEST_COPY_INPUTS");  // (tests: the other path)
   if (const char *e = std::getenv("ECHO_COMPOSE_KERNEL")) {  // tuning and tests: force a compose kernel
     const std::string k(e);
-    c->kernel_choice = k == "direct" ? 1 : k == "staged" ? 2 : k == "pipelined" ? 3 : k == "dataflow" ? 4 : 0;
+    c->kernel_choice = k == "direct" ? 1 : k == "staged" ? 2 : k == "levelled" || k == "pipelined" ? 3 : k == "dataflow" ? 4 : 0;  // ("pipelined": an earlier name)
   }
   // device waits give up after 2 s (tests shorten this and inject a level that never arrives)
   int clock_khz = 0;
@@ -2315,7 +2315,6 @@ int echo_compose(echo_ctx *c, const echo_compose_opts *opts) {
     o.cq_ops = c->cq_ops;
     o.lq_off = civ == ECHO_COMM_LAUNCH ? c->lq_off : nullptr;
     o.lq_ops = c->lq_ops;
-    o.kcl = c->kcl;
     o.f = f_prev;
     o.dur = c->dur;
     o.cd_used = cd_used;

@@ -207,7 +207,6 @@ struct OverlapArgs {
   // launch conditions of each entry of cq_ops on its rank (CSR); null: a comm op's
   // interval is its execution [start, finish), else [latest of them, finish)
   const int32_t *lq_off, *lq_ops;
-  const uint8_t *kcl;      // [V]
   const int64_t *f;        // finish times of the last pass
   const int64_t *dur;      // original durations
   const int64_t *cd_used;  // candidates' durations in the last pass (compact), or null: the original ones

@@ -51,11 +51,14 @@ def test_chain_and_join_edges_bit_exact(sigma, ranks, monkeypatch):
     g = _joins(ranks, [1, 3, 4, 5, 7, 8, 9] + ([63, 64, 65, 130] if ranks < 100 else [12]))
     rng = np.random.default_rng(100 * sigma + ranks)
     with Echo(0) as e:
+        e.set_profiling(True)
         for S in (sigma, 2 * sigma + 1):
             sc = SG.random_scenarios(rng, g, S, max_dur=20_000)
             for refine, model, interval in ((0, 0, 0), (1, 0, 0), (2, 1, 1)):
                 got = run_gpu(g, sc, refine, ctx=e, overlap_model=model, comm_interval=interval)
                 assert got["info"]["sigma"] == sigma
+                # (a plan that does not fit takes the staged composer, which has a name of its own)
+                assert {k for k in e.read_profile() if k.startswith("compose")} == {"compose"} | ({"compose_adjusted"} if refine else set())
                 want = oracle.compose(g, sc, refine_passes=refine, overlap_model=model, comm_interval=interval)
                 assert_same(got, want, g, refine)
 
@@ -70,6 +73,7 @@ def test_debug_bounds_of_every_block_width(sigma, monkeypatch):
     graphs = [_joins(11, [1, 3, 64, 65]), _joins(150, [1, 9, 12])]
     graphs += [SG.random_graph(rng, int(rng.integers(20, 300)), max_ranks=5, max_streams=8, p_edge=0.03) for _ in range(4)]
     with Echo(0) as e:
+        e.set_profiling(True)
         for g in graphs:
             sc = SG.random_scenarios(rng, g, sigma + 1, max_dur=20_000)
             for refine, model, interval in ((0, 0, 0), (2, 1, 1)):
@@ -77,6 +81,7 @@ def test_debug_bounds_of_every_block_width(sigma, monkeypatch):
                 e.load_scenarios(sc)
                 e.estimate_collectives()
                 e.compose(refine_passes=refine, overlap_model=model, comm_interval=interval, debug_bounds=True)
+                assert "compose" in e.read_profile()
                 st, fn = e.read_times()
                 got = dict(start=st, finish=fn, makespan=e.read_makespan(), cc=e.read_cc(), ov=e.read_overlap())
                 assert_same(got, oracle.compose(g, sc, refine_passes=refine, overlap_model=model, comm_interval=interval), g, refine)

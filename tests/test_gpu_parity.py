@@ -515,9 +515,9 @@ def test_gpt175b_1024_ranks_full_batch_bit_exact():
 @pytest.mark.parametrize("sigma", ["1", "2", "4", "8", "16"])
 @pytest.mark.parametrize("kernel", ["direct", "staged", "pipelined"])
 def test_every_compose_variant_bit_exact(sigma, kernel, monkeypatch):
-    # the three compose kernels (global-memory, cp.async-staged, bulk-copy pipelined;
-    # the pipelined one needs an even block width) at every scenario-block width,
-    # with full and partial scenario blocks
+    # the three compose kernels (global-memory, cp.async-staged, and the levelled one of
+    # warp roles, "pipelined") at every scenario-block width, with full and partial
+    # scenario blocks
     monkeypatch.setenv("ECHO_SIGMA", sigma)
     monkeypatch.setenv("ECHO_COMPOSE_KERNEL", kernel)
     c = W.config("gpt1.3b")
@@ -616,8 +616,8 @@ def test_dataflow_bounded_wait_reports_timeout(monkeypatch):
 
 
 def test_bounded_wait_reports_timeout(monkeypatch):
-    # failure detection without a GPU fault: the producer of the pipelined kernel
-    # never fills one segment level, every consumer's bounded wait gives up after
+    # failure detection without a GPU fault: the copy warps of the levelled composer
+    # never fill one step, every consumer's bounded wait gives up after
     # 20 ms, the block records the timeout and exits, and the host reports it
     c = W.config("gpt1.3b")
     g = W.build_gpt_graph(c)
