@@ -10,6 +10,8 @@ namespace echo {
 
 namespace {
 
+constexpr int kDirectSmem = 200 * 1024;  // most shared memory of a block of the direct kernel
+
 // ---------------------------------------------------------------------------------
 // B2: compose pass.  One thread block owns a block of SIGMA scenarios and walks
 // the graph segment level by segment level; scenarios never interact, so only
@@ -450,7 +452,7 @@ cudaError_t launch_compose_t(const ComposeArgs &a, cudaStream_t st) {
   dim3 grid((a.S + SIGMA - 1) / SIGMA);
   if (in_smem) {
     auto k = compose_direct_kernel<SIGMA, true>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kDirectSmem);  // (the same for all contexts)
     if (e != cudaSuccess) return e;
     k<<<grid, kComposeThreads, smem, st>>>(a);
   } else {
@@ -463,7 +465,7 @@ cudaError_t launch_compose_t(const ComposeArgs &a, cudaStream_t st) {
 template <int SIGMA, int THREADS>
 cudaError_t launch_staged_t(const StagedArgs &a, const StagedPlan &plan, cudaStream_t st) {
   auto k = compose_staged_kernel<SIGMA, THREADS>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_limit);
   if (e != cudaSuccess) return e;
   dim3 grid((a.S + SIGMA - 1) / SIGMA);
   k<<<grid, THREADS, plan.smem, st>>>(a);
@@ -475,7 +477,7 @@ cudaError_t launch_staged_t(const StagedArgs &a, const StagedPlan &plan, cudaStr
 size_t compose_smem_bytes(int32_t n_queues, int sigma, bool *frontier_in_smem) {
   size_t fr = (size_t)n_queues * sigma * sizeof(int64_t);
   size_t base = (size_t)sigma * sizeof(int64_t);
-  bool in = fr + base <= (size_t)200 * 1024;
+  bool in = fr + base <= (size_t)kDirectSmem;
   if (frontier_in_smem) *frontier_in_smem = in;
   return in ? fr + base : base;
 }

@@ -351,10 +351,12 @@ bool dataflow_fits(int64_t n_warps, int32_t n_streams, int32_t wpb, int device) 
   int sms = 0, coop = 0, per_sm0 = 0, per_sm1 = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
-  const size_t smem = dataflow_smem_bytes(n_streams, wpb);
-  if (cudaFuncSetAttribute(compose_dataflow_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+  // (The limit belongs to the kernel, not to a context: the same for all, 100 KB, so that no
+  // context or thread lowers it below another's launch.)
+  const size_t smem = dataflow_smem_bytes(n_streams, wpb), most = dataflow_smem_bytes(kMaxStreams, kDfMaxWarpsPerBlock);
+  if (cudaFuncSetAttribute(compose_dataflow_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) !=
           cudaSuccess ||
-      cudaFuncSetAttribute(compose_dataflow_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+      cudaFuncSetAttribute(compose_dataflow_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) !=
           cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm0, compose_dataflow_kernel<false>, 32 * wpb, smem) !=
           cudaSuccess ||

@@ -2165,6 +2165,7 @@ int echo_load_scenarios(echo_ctx *c, const echo_scen_desc *sc) {
       c->plan = plan_steps(B, sigma, staged_smem(c), c->steps);
     }
     // (threads of a staged block; may be overridden for tuning)
+    c->plan.smem_limit = level_smem(c);
     c->plan.threads = sigma == 16 ? 1024 : sigma == 8 ? 512 : sigma == 4 ? 256 : 512;
     if (const char *e = std::getenv("ECHO_STAGED_THREADS")) c->plan.threads = std::atoi(e);
     if (c->plan.ok) {

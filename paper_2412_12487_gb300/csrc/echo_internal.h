@@ -114,6 +114,7 @@ struct StagedPlan {
   int threads = 512;       // threads per block
   int vring_log2 = 0, dring_log2 = 0, rring_log2 = 0;  // sizes (segments, rows, words)
   size_t smem = 0;
+  size_t smem_limit = 0;   // what the device gives a block: the kernel's limit, the same for every context
 };
 
 // Shared-memory layout of the staged kernel (byte offsets).  Every region starts

@@ -135,3 +135,31 @@ def test_choice_among_composers_that_exist(lengths, S, sigma, ran):
             assert e.info()["sigma"] == sigma
             assert [k for k in e.read_profile() if k.startswith("compose")][0] == ran
             assert_same(got, oracle.compose(g, sc, threads=8), g)
+
+
+@pytest.mark.parametrize("kernel", ["dataflow", "staged", "direct", "levelled"])
+def test_contexts_with_different_shared_memory(kernel, monkeypatch):
+    """Blocks of two contexts need different amounts of shared memory; neither's batches lower the other's limit."""
+    monkeypatch.setenv("ECHO_COMPOSE_KERNEL", kernel)
+    shapes = [W.GPTConfig("case", layers=4, hidden=1024, heads=8, seq=512, tp=tp, pp=2, dp=2, microbatches=4, virtual_stages=v, n_scen=7)
+              for tp, v in ((8, 2), (2, 1))]  # blocks of 8 ranks with 8 timelines; of 2 with fewer
+    batches = []
+    for c in shapes:
+        g = W.build_gpt_graph(c)
+        sc = W.make_scenarios(g, c, n_scen=7)
+        batches.append((g, sc, oracle.compose(g, sc)))
+    contexts = [Echo(0) for _ in batches]
+    try:
+        for e, (g, sc, _) in zip(contexts, batches):
+            e.load_graph(g)
+            e.load_scenarios(sc)
+        for order in ((0, 1), (1, 0), (0, 1)):
+            for i in order:
+                contexts[i].load_scenarios(batches[i][1])
+            for i in order:
+                contexts[i].estimate_collectives()
+                contexts[i].compose()
+                assert np.array_equal(contexts[i].read_times()[1], batches[i][2].finish)
+    finally:
+        for e in contexts:
+            e.close()
